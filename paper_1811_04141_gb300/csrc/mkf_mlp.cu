@@ -57,64 +57,120 @@ __global__ void __launch_bounds__(128) forward_kernel(const uint16_t *wb, const 
     logit[s] = z;
 }
 
-// Per sample: forward, d(loss)/d(logit) = (sigmoid(z) - y) / n, the hidden
-// activations H and the pre-activation gradient dA, and the sample's loss.
-__global__ void __launch_bounds__(128) sample_grad_kernel(const uint16_t *wb, const float *feat, const float *label,
-                                                          int n, float *H, float *dA, float *g, float *ls) {
-    __shared__ float ws[kP];
-    load_weights(wb, ws);
-    const int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n) return;
-    float x[kIn];
-#pragma unroll
-    for (int k = 0; k < kIn; ++k) x[k] = feat[(int64_t)s * kIn + k];
-    float z = ws[kOffB2];
-    for (int j = 0; j < kHid; ++j) {
-        float a = ws[kOffB1 + j];
-#pragma unroll
-        for (int k = 0; k < kIn; ++k) a = fmaf(ws[j * kIn + k], x[k], a);
-        const float h = fmaxf(a, 0.f);
-        H[(int64_t)s * kHid + j] = h;
-        dA[(int64_t)s * kHid + j] = a > 0.f ? 1.f : 0.f;  // ReLU mask, scaled below
-        z = fmaf(ws[kOffW2 + j], h, z);
-    }
-    const float y = label[s];
-    const float e = expf(-fabsf(z));
-    const float sig = z >= 0.f ? 1.f / (1.f + e) : e / (1.f + e);
-    const float gs = (sig - y) / static_cast<float>(n);
-    g[s] = gs;
-    ls[s] = fmaxf(z, 0.f) - z * y + log1pf(e);
-    for (int j = 0; j < kHid; ++j) dA[(int64_t)s * kHid + j] *= gs * ws[kOffW2 + j];
-}
+// Gradient of one chunk of samples, reduced over the chunk: block (x, y) takes
+// chunk y and the kSlice hidden units of slice x.  First one thread per sample:
+// forward, d(loss)/d(logit) = (sigmoid(z) - y) / n, the sample's loss and, for
+// the slice's units, the activations and the pre-activation gradients, all kept
+// in shared memory; then one thread per parameter of the slice sums its samples
+// in order (compensated).  wf: FP32 weights, rounded here as to_bf16 does, or
+// nullptr to take wb.
+// Bound: latency (4096 samples are 16 chunks: too few blocks to fill the chip,
+// and a chunk's compensated sum is 256 dependent steps of four additions, 2 us).
+// Every slice therefore repeats the chunk's forward pass (1 us) so that 8 blocks
+// work on a chunk, and nothing per sample goes through global memory: the
+// activations and gradients written there by one kernel and read back by the
+// next, one load per addition, made a training step of 4096 samples take 108 us
+// (four kernels; 16.3 us with this one and finish_kernel, bit for bit the same).
+constexpr int kSlice = 8;
+constexpr int kSlices = kHid / kSlice;
+constexpr int kRow = kChunk + 4;  // a row of the transposed tiles: 16-byte aligned, rows 4 banks apart
+constexpr int kSliceParams = kSlice * (kIn + 2);
+static_assert(kHid % kSlice == 0 && kSliceParams + 2 <= kChunk && kChunk % 4 == 0, "one thread per parameter");
 
-// Partial sums over one chunk of samples for every parameter (+ the loss),
-// compensated (Kahan) summation in sample order.
-__global__ void __launch_bounds__(128) chunk_reduce_kernel(const float *feat, const float *H, const float *dA,
-                                                           const float *g, const float *ls, int n, float *part) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;  // parameter index, kP = the loss
-    if (p > kP) return;
-    const int s0 = blockIdx.y * kChunk, s1 = min(n, s0 + kChunk);
+// Compensated (Kahan) sum in the order of the calls.
+struct KahanSum {
     float sum = 0.f, comp = 0.f;
-    for (int s = s0; s < s1; ++s) {
-        float t;
-        if (p < kOffB1) {
-            const int j = p / kIn, k = p - j * kIn;
-            t = dA[(int64_t)s * kHid + j] * feat[(int64_t)s * kIn + k];
-        } else if (p < kOffW2) {
-            t = dA[(int64_t)s * kHid + (p - kOffB1)];
-        } else if (p < kOffB2) {
-            t = g[s] * H[(int64_t)s * kHid + (p - kOffW2)];
-        } else if (p == kOffB2) {
-            t = g[s];
-        } else {
-            t = ls[s];
-        }
+    __device__ __forceinline__ void add(float t) {
         const float yv = t - comp;
         const float tt = sum + yv;
         comp = (tt - sum) - yv;
         sum = tt;
     }
-    part[(int64_t)blockIdx.y * (kP + 1) + p] = sum;
+};
+
+__global__ void __launch_bounds__(kChunk) chunk_grad_kernel(const uint16_t *wb, const float *wf, const float *feat,
+                                                            const float *label, int n, float *part) {
+    __shared__ __align__(16) float xs[kIn * kRow];     // features, [k][sample]
+    __shared__ __align__(16) float hs[kSlice * kRow];  // the slice's activations, [unit][sample]
+    __shared__ __align__(16) float ds[kSlice * kRow];  // the slice's pre-activation gradients
+    __shared__ __align__(16) float gs[kChunk];
+    __shared__ __align__(16) float ls[kChunk];
+    __shared__ __align__(16) float ws[kP + 3];
+    const int tid = threadIdx.x;
+    const int j0 = blockIdx.x * kSlice;
+    const int s0 = blockIdx.y * kChunk, ns = min(kChunk, n - s0);
+    for (int i = tid; i < kP; i += kChunk) ws[i] = from_bf16(wf ? to_bf16(wf[i]) : wb[i]);
+    for (int i = tid; i < ns * kIn; i += kChunk) {
+        const int s = i / kIn, k = i - s * kIn;
+        xs[k * kRow + s] = feat[(int64_t)s0 * kIn + i];
+    }
+    __syncthreads();
+    if (tid < ns) {
+        float x[kIn];
+#pragma unroll
+        for (int k = 0; k < kIn; ++k) x[k] = xs[k * kRow + tid];
+        float z = ws[kOffB2];
+#pragma unroll 4
+        for (int j = 0; j < kHid; ++j) {
+            const float4 *row = reinterpret_cast<const float4 *>(ws + j * kIn);
+            const float4 r0 = row[0], r1 = row[1], r2 = row[2];
+            const float wr[kIn] = {r0.x, r0.y, r0.z, r0.w, r1.x, r1.y, r1.z, r1.w, r2.x, r2.y, r2.z, r2.w};
+            float a = ws[kOffB1 + j];
+#pragma unroll
+            for (int k = 0; k < kIn; ++k) a = fmaf(wr[k], x[k], a);
+            const float h = fmaxf(a, 0.f);
+            const int jj = j - j0;
+            if (jj >= 0 && jj < kSlice) {
+                hs[jj * kRow + tid] = h;
+                ds[jj * kRow + tid] = a > 0.f ? 1.f : 0.f;  // ReLU mask, scaled below
+            }
+            z = fmaf(ws[kOffW2 + j], h, z);
+        }
+        const float y = label[s0 + tid];
+        const float e = expf(-fabsf(z));
+        const float sig = z >= 0.f ? 1.f / (1.f + e) : e / (1.f + e);
+        const float g = (sig - y) / static_cast<float>(n);
+        gs[tid] = g;
+        ls[tid] = fmaxf(z, 0.f) - z * y + log1pf(e);
+#pragma unroll
+        for (int jj = 0; jj < kSlice; ++jj) ds[jj * kRow + tid] *= g * ws[kOffW2 + j0 + jj];
+    }
+    __syncthreads();
+    // the slice's parameters: W1 rows, b1, w2; slice 0 also takes b2 and the loss
+    if (tid >= kSliceParams + (blockIdx.x == 0 ? 2 : 0)) return;
+    const float *a, *b = nullptr;  // the sum of a[s] b[s], or of a[s]
+    int p;
+    if (tid < kSlice * kIn) {
+        const int jj = tid / kIn, k = tid - jj * kIn;
+        a = ds + jj * kRow;
+        b = xs + k * kRow;
+        p = (j0 + jj) * kIn + k;
+    } else if (tid < kSlice * (kIn + 1)) {
+        const int jj = tid - kSlice * kIn;
+        a = ds + jj * kRow;
+        p = kOffB1 + j0 + jj;
+    } else if (tid < kSliceParams) {
+        const int jj = tid - kSlice * (kIn + 1);
+        a = gs;
+        b = hs + jj * kRow;
+        p = kOffW2 + j0 + jj;
+    } else {
+        a = tid == kSliceParams ? gs : ls;
+        p = tid == kSliceParams ? kOffB2 : kP;
+    }
+    KahanSum acc;
+    int s = 0;
+    for (; s + 4 <= ns; s += 4) {
+        const float4 u = *reinterpret_cast<const float4 *>(a + s);
+        float4 v = make_float4(1.f, 1.f, 1.f, 1.f);
+        if (b) v = *reinterpret_cast<const float4 *>(b + s);
+        acc.add(__fmul_rn(u.x, v.x));
+        acc.add(__fmul_rn(u.y, v.y));
+        acc.add(__fmul_rn(u.z, v.z));
+        acc.add(__fmul_rn(u.w, v.w));
+    }
+    for (; s < ns; ++s) acc.add(__fmul_rn(a[s], b ? b[s] : 1.f));
+    part[(int64_t)blockIdx.y * (kP + 1) + p] = acc.sum;
 }
 
 // Sum the chunk partials in chunk order; optionally apply Adam.
@@ -122,13 +178,10 @@ __global__ void __launch_bounds__(128) finish_kernel(const float *part, int nchu
                                                      float *w, float *m, float *v, int t, mkf_adam hp, uint16_t *wb) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p > kP) return;
-    float sum = 0.f, comp = 0.f;
-    for (int c = 0; c < nchunks; ++c) {
-        const float yv = part[(int64_t)c * (kP + 1) + p] - comp;
-        const float tt = sum + yv;
-        comp = (tt - sum) - yv;
-        sum = tt;
-    }
+    KahanSum acc;
+#pragma unroll 8
+    for (int c = 0; c < nchunks; ++c) acc.add(part[(int64_t)c * (kP + 1) + p]);
+    const float sum = acc.sum;
     if (p == kP) {
         if (loss) *loss = sum / static_cast<float>(n);
         return;
@@ -147,23 +200,16 @@ __global__ void __launch_bounds__(128) finish_kernel(const float *part, int nchu
     }
 }
 
+// wb: bfloat16 weights, or nullptr to round the FP32 weights w (a training step).
 mkf_status run_grad(mkf_ctx *ctx, const uint16_t *wb, const float *feat, const float *label, int n, float *grad,
                     float *loss, float *w, float *m, float *v, int t, const mkf_adam *hp, uint16_t *wb_out) {
     const int nchunks = (n + kChunk - 1) / kChunk;
-    const size_t floats = (size_t)n * kHid * 2 + (size_t)n * 2 + (size_t)nchunks * (kP + 1);
     void *scratch = nullptr;
-    mkf_status st = mkf_scratch(ctx, floats * sizeof(float), &scratch);
+    mkf_status st = mkf_scratch(ctx, (size_t)nchunks * (kP + 1) * sizeof(float), &scratch);
     if (st != MKF_OK) return st;
-    float *H = static_cast<float *>(scratch);
-    float *dA = H + (size_t)n * kHid;
-    float *g = dA + (size_t)n * kHid;
-    float *ls = g + n;
-    float *part = ls + n;
+    float *part = static_cast<float *>(scratch);
     cudaStream_t s = ctx->stream;
-    sample_grad_kernel<<<(n + 127) / 128, 128, 0, s>>>(wb, feat, label, n, H, dA, g, ls);
-    MKF_CUDA_TRY(cudaGetLastError());
-    dim3 grid((kP + 1 + 127) / 128, nchunks);
-    chunk_reduce_kernel<<<grid, 128, 0, s>>>(feat, H, dA, g, ls, n, part);
+    chunk_grad_kernel<<<dim3(kSlices, nchunks), kChunk, 0, s>>>(wb, wb ? nullptr : w, feat, label, n, part);
     MKF_CUDA_TRY(cudaGetLastError());
     mkf_adam h = hp ? *hp : mkf_adam{0.f, 0.f, 0.f, 0.f};
     finish_kernel<<<(kP + 1 + 127) / 128, 128, 0, s>>>(part, nchunks, n, grad, loss, w, m, v, t, h, wb_out);
@@ -208,8 +254,5 @@ extern "C" mkf_status mkf_mlp_train_step(mkf_ctx *ctx, const float *feat, const 
     if (!ctx || !feat || !label || !w || !m || !v || !hp || !w_bf16 || n < 1 || t < 1) return MKF_ERR_ARG;
     DeviceGuard g(ctx->device);
     if (!g.ok) return MKF_ERR_CUDA;
-    // bfloat16 copy of the current masters for the forward pass
-    to_bf16_kernel<<<(MKF_MLP_PARAMS + 255) / 256, 256, 0, ctx->stream>>>(w, w_bf16, MKF_MLP_PARAMS);
-    MKF_CUDA_TRY(cudaGetLastError());
-    return run_grad(ctx, w_bf16, feat, label, n, nullptr, loss, w, m, v, t, hp, w_bf16);
+    return run_grad(ctx, nullptr, feat, label, n, nullptr, loss, w, m, v, t, hp, w_bf16);
 }
