@@ -75,6 +75,10 @@ struct FindArgs {
     // the seed kernel writes each seed's key and place, order_scatter_kernel
     // the order the finder's warps take the seeds in
     int32_t *order_key, *order_pos, *order_counts;
+    // seeds left to find_wide_kernel (or nullptr: none are): entries seed + 1,
+    // zero until written; how many were added and how many taken
+    int32_t *wide_list, *wide_count, *wide_next;
+    int32_t wide_bins;  // bins of a wide window
 };
 
 // Seeds are taken by the finder grouped by event and by the |eta| of their
@@ -311,7 +315,20 @@ struct Expansion {
     int nlist;      // compatible hits kept (at most N), sorted by (chi2, hit index)
     int n_compat;   // all compatible hits
     float cot;      // cot(theta) before the move
+    bool wide;      // not searched: the window is too wide for one lane
 };
+
+// With scattering and energy loss a few seeds in a hundred get candidates whose
+// windows span much of a layer (thousands of hits).  One lane scanning them
+// takes up to 3 ms while the rest of the call takes 1 ms (8 dense events with
+// material, N = 10: 3.7 ms with and 1.1 ms without the 3000 widest of 48 000
+// seeds), so the variants with material leave a seed to find_wide_kernel, which
+// gives every candidate several lanes, as soon as one of its windows holds about
+// this many hits (A.wide_bins bins at the call's mean occupancy).  Measured on
+// that call and on a learned cascade over 16 such events: 77 hits 2.2 / 3.3 ms,
+// 128 1.9 / 2.6, 205 1.8 / 2.3, 320 1.8 / 2.3; by phi bins alone (16 to 48)
+// 1.8-2.1 / 2.4-2.9.
+constexpr int kWideHits = 256;
 
 // One candidate to its next layer: next-layer choice, propagation and
 // covariance transport, S^-1 and H C, the bins of the chi2 window, and the
@@ -320,11 +337,16 @@ struct Expansion {
 // arrays in the seed kernel).  p, lo, C move onto the layer; a candidate with no
 // layer left is marked done.  kPhys: 0 uniform field, 1 material effects,
 // 2 parameterised field (Runge-Kutta propagation) and material effects.
-template <int kPhys>
+// kLeave: a wide window is not searched but marked (X.wide).  kShared: the
+// candidate is held by `lanes` lanes, which share its window: lane `sub` takes
+// the phi bins sub, sub + lanes, ... counted from the middle of the window
+// outwards (the best hits come first and the lists settle) and keeps a list of
+// its own.
+template <int kPhys, bool kLeave, bool kShared>
 __device__ __forceinline__ void expand(const FindArgs &A, const Geom &G, int ev, unsigned long long mask, int dir,
                                        int N, float cut, float p[6], Lo &lo, float C[21], Book &bk, Innov &I,
                                        uint32_t &status, int &c_cl, int &c_ht, float *lchi, int *lorig, float *lu,
-                                       float *lv, int ls, Expansion &X) {
+                                       float *lv, int ls, Expansion &X, int sub = 0, int lanes = 1) {
     float sphi, cphi;
     sincos_pair(p[4], lo.phi, sphi, cphi);
     const float cot = cot_pair(p[5], lo.th);
@@ -332,6 +354,7 @@ __device__ __forceinline__ void expand(const FindArgs &A, const Geom &G, int ev,
     X.searched = false;
     X.nlist = 0;
     X.n_compat = 0;
+    X.wide = false;
     float s = 0.f;
     const float kbl = kPhys == 2 ? G.kb * bz_factor(G.alpha, p[0], p[1], p[2]) : G.kb;
     const int l = finite_state(p) ? next_layer(G, kbl, mask, p, lo, sphi, cphi, cot, dir, bk.ncyl, bk.ndsk, s) : -2;
@@ -382,6 +405,10 @@ __device__ __forceinline__ void expand(const FindArgs &A, const Geom &G, int ev,
     const float zhi_f = fminf(fmaxf(floorf((zc + wz - Ld.lo) * Ld.zr_scale), 0.f), Ld.nzr - 1.f);
     const int zb_lo = static_cast<int>(zlo_f), zb_hi = static_cast<int>(zhi_f);
     const int ebase = ev * G.bins_per_event + Ld.bin_base;
+    if (kLeave && A.wide_list && nphib * (zb_hi - zb_lo + 1) >= A.wide_bins) {
+        X.wide = true;
+        nphib = 0;
+    }
     int nlist = 0, n_compat = 0;
     // Loads run one ahead: the offsets of the next phi bin load while this
     // bin's hits are tested, and each hit record while the one before it is
@@ -389,8 +416,9 @@ __device__ __forceinline__ void expand(const FindArgs &A, const Geom &G, int ev,
     // time: -25 % for the widest-window seeds with material, -10 % for the
     // whole material workload, no change without material).
     // the hit range [k0, k1) of the window's z (or r) bins in phi bin i
+    const int half = nphib >> 1;
     auto bin_range = [&](int i, int &k0, int &k1) {
-        int pb = pb_lo + i;
+        int pb = pb_lo + (kShared ? half + ((i & 1) ? -((i + 1) >> 1) : (i >> 1)) : i);
         if (pb < 0) pb += Ld.nphi;
         else if (pb >= Ld.nphi) pb -= Ld.nphi;
         const int bin = ebase + pb * Ld.nzr;
@@ -398,10 +426,11 @@ __device__ __forceinline__ void expand(const FindArgs &A, const Geom &G, int ev,
         k1 = A.offsets[bin + zb_hi + 1];
     };
     int nk0 = 0, nk1 = 0;
-    if (nphib > 0) bin_range(0, nk0, nk1);
-    for (int i = 0; i < nphib; ++i) {
+    const int first = kShared ? sub : 0, stride = kShared ? lanes : 1;
+    if (first < nphib) bin_range(first, nk0, nk1);
+    for (int i = first; i < nphib; i += stride) {
         const int k0 = nk0, k1 = nk1;
-        if (i + 1 < nphib) bin_range(i + 1, nk0, nk1);
+        if (i + stride < nphib) bin_range(i + stride, nk0, nk1);
         float4 nhr = k0 < k1 ? A.rec[k0] : make_float4(0.f, 0.f, 0.f, 0.f);
         for (int k = k0; k < k1; ++k) {
             const float4 hr = nhr;
@@ -588,7 +617,7 @@ __global__ void __launch_bounds__(128) seed_kernel(const __grid_constant__ FindA
         float lchi[MKF_MAX_NBEST], lu[MKF_MAX_NBEST], lv[MKF_MAX_NBEST];
         int lorig[MKF_MAX_NBEST];
         Expansion X;
-        expand<kPhys>(A, G, ev, mask, dir, N, A.cut, p, lo, C, bk, I, status, c_cl, c_ht, lchi, lorig, lu, lv, 1, X);
+        expand<kPhys, false, false>(A, G, ev, mask, dir, N, A.cut, p, lo, C, bk, I, status, c_cl, c_ht, lchi, lorig, lu, lv, 1, X);
         nlist = X.nlist;
         searched = X.searched;
         nbeam = min(searched ? nlist + 1 : 1, N);
@@ -634,6 +663,60 @@ __global__ void __launch_bounds__(128) seed_kernel(const __grid_constant__ FindA
     for (int k = 0; k < 3; ++k) B[(SF_HITS + k) * (int64_t)n + t] = __int_as_float(hidx[k]);
 }
 
+// The outputs of a seed from its best candidate (rank 0): state, hit list
+// walked back through the step history (row st, column base + rank), counters.
+__device__ __forceinline__ void write_track(const FindArgs &A, int seed, int ev, uint32_t status, bool live,
+                                            const Book &bk, float p[6], const Lo &lo, const float C[21], float chi2,
+                                            int sh0, int sh1, int sh2, const uint32_t *hist, int hstride, int base,
+                                            int step, int c_cl, int c_ht, int c_up) {
+    const int n = A.n_seeds;
+    const bool ok = !(status & MKF_ST_BADSEED) && live;
+    int nout = 0;
+    if (ok) {
+        const int shs[3] = {sh0, sh1, sh2};
+        for (int k = 0; k < 3 && nout < A.max_out; ++k) A.out_hits[(int64_t)(nout++) * n + seed] = shs[k];
+        // the hits the finder added (the candidate's count beyond its three
+        // seed hits), written from the last backwards while the history is
+        // walked back from the best candidate
+        const int cnt = bk.nh - 3;
+        int pos = nout + cnt - 1;
+        int r = 0;
+        for (int st = step - 1; st >= 0; --st) {
+            const uint32_t rec = hist[st * hstride + base + r];
+            const uint32_t code = rec & kHitMask;
+            if (code < kCodeMiss) {
+                if (pos < A.max_out) A.out_hits[(int64_t)pos * n + seed] = static_cast<int>(code);
+                --pos;
+            }
+            r = static_cast<int>(rec >> 28);
+        }
+        if (nout + cnt > A.max_out) status |= MKF_ST_TRUNC;
+        nout = min(nout + cnt, A.max_out);
+        if (bk.missstop) status |= MKF_ST_MISSSTOP;
+        if (!finite_state(p) || !isfinite(chi2)) status |= MKF_ST_NONFINITE;
+    }
+    for (int k = nout; k < A.max_out; ++k) A.out_hits[(int64_t)k * n + seed] = -1;
+    const float nanv = __int_as_float(0x7fc00000);
+    p[0] += lo.x;
+    p[1] += lo.y;
+    p[2] += lo.z;
+    p[4] += lo.phi;
+    p[5] += lo.th;
+#pragma unroll
+    for (int i = 0; i < 6; ++i) A.out_par[(int64_t)i * n + seed] = ok ? p[i] : nanv;
+#pragma unroll
+    for (int k = 0; k < 21; ++k) A.out_cov[(int64_t)k * n + seed] = ok ? C[k] : nanv;
+    A.out_chi2[seed] = ok ? chi2 : nanv;
+    A.out_nhits[seed] = ok ? bk.nh : 0;
+    A.out_status[seed] = status;
+    if (A.counters) {
+        A.counters[seed] = c_cl;
+        A.counters[(int64_t)n + seed] = c_ht;
+        A.counters[2 * (int64_t)n + seed] = c_up;
+    }
+    if (A.event_times && ev >= 0 && ev < A.n_events) atomicMax(&A.event_times[ev], globaltimer_ns());
+}
+
 // kLearned: the variant with learned pruning and the feature dump compiled in;
 // the plain finder is built without them.  kPhys: 0 uniform field; 1 the
 // material effects compiled in (selected when any layer has material); 2 the
@@ -643,6 +726,8 @@ __global__ void __launch_bounds__(128) seed_kernel(const __grid_constant__ FindA
 // not for the parameterised field), or 0 for N taken from the arguments.
 template <bool kLearned, int kPhys, int kN>
 __global__ void __launch_bounds__(256, 2) find_kernel(const __grid_constant__ FindArgs A) {
+    // (learned: the cascade's best-hit pass)
+    constexpr bool kLeave = kPhys >= 1 && (!kLearned || kN == 1);
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ Geom SG;
     __shared__ float WS[MKF_MLP_PARAMS];
@@ -686,7 +771,13 @@ __global__ void __launch_bounds__(256, 2) find_kernel(const __grid_constant__ Fi
         int grp = 0;
         if (lane == 0) grp = atomicAdd(A.work_counter, 1);
         grp = __shfl_sync(kFull, grp, 0);
-        if (grp >= n_groups) break;
+        if (grp >= n_groups) {
+#ifdef __CUDACC__
+            // find_wide_kernel may start where blocks of this one have ended
+            if (kLeave) asm volatile("griddepcontrol.launch_dependents;");
+#endif
+            break;
+        }
         const int li = grp * spw + slot;
         int seed = li;
         bool has_seed = lane_used && li < n_call;
@@ -828,10 +919,22 @@ __global__ void __launch_bounds__(256, 2) find_kernel(const __grid_constant__ Fi
             const bool active = live && !bk.done;
             if (!__any_sync(kFull, active)) break;  // every candidate of the warp has finished
             // ---- 1. expansion: next layer, propagation, window search
-            Expansion X{-1, false, 0, 0, 0.f};
+            Expansion X{-1, false, 0, 0, 0.f, false};
             if (active) {
-                expand<kPhys>(A, G, ev, mask, dir, N, cut, p, lo, C, bk, I, status, c_cl, c_ht, lchi + lane, lorig + lane,
-                       lu + lane, lv + lane, 32, X);
+                expand<kPhys, kLeave, false>(A, G, ev, mask, dir, N, cut, p, lo, C, bk, I, status, c_cl, c_ht,
+                                             lchi + lane, lorig + lane, lu + lane, lv + lane, 32, X);
+            }
+            if (kLeave && A.wide_list) {
+                // a seed with a wide window ends here, without output: it is
+                // found from its start by find_wide_kernel
+                const unsigned wide = __ballot_sync(kFull, X.wide);
+                if (wide && lane_used && has_seed && ((wide >> base) & (0xffffffffu >> (32 - N)))) {
+                    if (rank == 0) A.wide_list[atomicAdd(A.wide_count, 1)] = seed + 1;
+                    has_seed = false;
+                    live = false;
+                    X.searched = false;
+                    X.nlist = 0;
+                }
             }
             // learned pruning / feature dump over the candidate's list (its N best
             // compatible hits); the MLP scores a list only when the candidate has
@@ -995,52 +1098,8 @@ __global__ void __launch_bounds__(256, 2) find_kernel(const __grid_constant__ Fi
         c_up = seg_sum(c_up, rank, N);
         status = seg_or(status, rank, N);
         if (has_seed && rank == 0) {
-            const int n = A.n_seeds;
-            const bool ok = !(status & MKF_ST_BADSEED) && live;
-            int nout = 0;
-            if (ok) {
-                const int shs[3] = {sh0, sh1, sh2};
-                for (int k = 0; k < 3 && nout < A.max_out; ++k) A.out_hits[(int64_t)(nout++) * n + seed] = shs[k];
-                // the hits the finder added (the candidate's count beyond its three
-                // seed hits), written from the last backwards while the history is
-                // walked back from the best candidate
-                const int cnt = bk.nh - 3;
-                int pos = nout + cnt - 1;
-                int r = 0;
-                for (int st = step - 1; st >= 0; --st) {
-                    const uint32_t rec = hist[st * 32 + base + r];
-                    const uint32_t code = rec & kHitMask;
-                    if (code < kCodeMiss) {
-                        if (pos < A.max_out) A.out_hits[(int64_t)pos * n + seed] = static_cast<int>(code);
-                        --pos;
-                    }
-                    r = static_cast<int>(rec >> 28);
-                }
-                if (nout + cnt > A.max_out) status |= MKF_ST_TRUNC;
-                nout = min(nout + cnt, A.max_out);
-                if (bk.missstop) status |= MKF_ST_MISSSTOP;
-                if (!finite_state(p) || !isfinite(chi2)) status |= MKF_ST_NONFINITE;
-            }
-            for (int k = nout; k < A.max_out; ++k) A.out_hits[(int64_t)k * n + seed] = -1;
-            const float nanv = __int_as_float(0x7fc00000);
-            p[0] += lo.x;
-            p[1] += lo.y;
-            p[2] += lo.z;
-            p[4] += lo.phi;
-            p[5] += lo.th;
-    #pragma unroll
-            for (int i = 0; i < 6; ++i) A.out_par[(int64_t)i * n + seed] = ok ? p[i] : nanv;
-    #pragma unroll
-            for (int k = 0; k < 21; ++k) A.out_cov[(int64_t)k * n + seed] = ok ? C[k] : nanv;
-            A.out_chi2[seed] = ok ? chi2 : nanv;
-            A.out_nhits[seed] = ok ? bk.nh : 0;
-            A.out_status[seed] = status;
-            if (A.counters) {
-                A.counters[seed] = c_cl;
-                A.counters[(int64_t)n + seed] = c_ht;
-                A.counters[2 * (int64_t)n + seed] = c_up;
-            }
-            if (A.event_times && ev >= 0 && ev < A.n_events) atomicMax(&A.event_times[ev], globaltimer_ns());
+            write_track(A, seed, ev, status, live, bk, p, lo, C, chi2, sh0, sh1, sh2, hist, 32, base, step, c_cl, c_ht,
+                        c_up);
         }
     }
 }
@@ -1151,6 +1210,324 @@ size_t find_smem_bytes(int n_layers, int n_best, int threads) {
 
 }  // namespace
 
+namespace {
+
+// Lanes that share a candidate of find_wide_kernel: a candidate's lanes sit in
+// one warp.
+__host__ __device__ constexpr int wide_lanes(int N) { return N == 1 ? 32 : 16; }
+__host__ __device__ constexpr int wide_threads(int N) { return (N * wide_lanes(N) + 31) / 32 * 32; }
+
+constexpr int kWideState = 56;  // words of a candidate handed to its children
+constexpr int kWideRanks = MKF_MAX_NBEST;
+
+size_t wide_smem_bytes(int n_layers, int N) {
+    const size_t words = (size_t)find_max_steps(n_layers) * kWideRanks + 4 * (size_t)N * wide_threads(N) +
+                         4 * (size_t)N * kWideRanks + (size_t)kWideState * kWideRanks + kWideRanks;
+    return words * 4;
+}
+
+// The next seed of the list, or -1: none, or the next entry is not written yet.
+__device__ __forceinline__ int next_wide(const FindArgs &A) {
+    const volatile int32_t *next = A.wide_next, *list = A.wide_list;
+    int n = *next;
+    while (n < A.n_seeds) {
+        const int e = list[n];
+        if (e == 0) return -1;
+        const int was = atomicCAS(A.wide_next, n, n + 1);
+        if (was == n) return e - 1;
+        n = was;
+    }
+    return -1;
+}
+
+// The finder for the seeds that find_kernel left because of a wide window (see
+// kWideHits): one block per seed, wide_lanes(N) lanes per candidate.  The lanes
+// of a candidate all hold its state and move it together (the same arithmetic
+// as in find_kernel, so the same bits); they share the phi bins of its window,
+// each with a list of its own, and the lists are merged by N rounds of a minimum
+// over (chi2, hit index).  The seed's N children are chosen by one warp with
+// find_kernel's keys and take their parents' states through shared memory.
+// Bound: the latency of a seed's chain of steps; a window of 4000 hits takes
+// 250 tests a lane instead of 4000 (8 lanes a candidate instead of 16: 10 %
+// slower), and the blocks of such seeds run side by side: the seed with the
+// widest windows takes 0.55 ms instead of 3.2 ms, the call above 1.8 ms instead
+// of 2.7 to 3.6 ms (by event sample).  Slower: the lanes of find_kernel's own
+// warp sharing one window after the other (2.5 ms; they are only three to a
+// candidate), or sharing the windows of a seed that a warp takes alone (2.4-2.8
+// ms).  The launch is a programmatic dependent one: its blocks
+// start where find_kernel's have ended, take the seeds listed by then, and wait
+// for find_kernel's end (griddepcontrol.wait) before they take the rest (0.2 ms less than one kernel
+// after the other).
+template <bool kLearned, int kPhys>
+__global__ void __launch_bounds__(256, 2) find_wide_kernel(const __grid_constant__ FindArgs A) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ Geom SG;
+    __shared__ float WS[kLearned ? MKF_MLP_PARAMS : 1];
+    __shared__ int s_item, s_got, s_cl, s_ht, s_up;
+    __shared__ uint32_t s_status;
+    const int tid = threadIdx.x, nt = blockDim.x;
+    {
+        const int *src = reinterpret_cast<const int *>(&A.G);
+        int *dst = reinterpret_cast<int *>(&SG);
+        for (int i = tid; i < static_cast<int>(sizeof(Geom) / sizeof(int)); i += nt) dst[i] = src[i];
+        if (kLearned)
+            for (int i = tid; i < MKF_MLP_PARAMS; i += nt)
+                WS[i] = __uint_as_float(static_cast<uint32_t>(A.mlp[i]) << 16);
+    }
+    const Geom &G = SG;
+    const int N = A.n_best, lanes = wide_lanes(N);
+    const int rank = tid / lanes, sub = tid - rank * lanes;
+    const bool lane_used = rank < N;
+    const bool lead = lane_used && sub == 0;
+    const int row = lane_used ? rank : 0;  // an in-bounds row for every lane
+    uint32_t *hist = reinterpret_cast<uint32_t *>(smem);
+    float *lchi = reinterpret_cast<float *>(hist + A.max_steps * kWideRanks);  // the lanes' lists [N][nt]
+    int *lorig = reinterpret_cast<int *>(lchi) + N * nt;
+    float *lu = lchi + 2 * N * nt, *lv = lchi + 3 * N * nt;
+    float *mchi = lchi + 4 * N * nt;  // the candidates' lists [N][kWideRanks]
+    int *morig = reinterpret_cast<int *>(mchi) + N * kWideRanks;
+    float *mu = mchi + 2 * N * kWideRanks, *mv = mchi + 3 * N * kWideRanks;
+    float *state = mchi + 4 * N * kWideRanks;  // [kWideRanks][kWideState]
+    int *sel = reinterpret_cast<int *>(state + kWideState * kWideRanks);
+    const float cut = A.cut;
+    bool last = false;  // find_kernel has ended: the list is complete
+    for (;;) {
+        __syncthreads();
+        if (tid == 0) {
+            s_item = next_wide(A);
+            s_cl = s_ht = s_up = 0;
+            s_status = 0;
+        }
+        __syncthreads();
+        const int seed = s_item;
+        if (seed < 0) {
+            if (last) break;
+            last = true;
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            continue;
+        }
+        const float *Bs = A.seedbuf;
+        const int64_t n = A.n_seeds;
+        const int ev = A.seed_event[seed];
+        const unsigned long long mask =
+            static_cast<unsigned long long>(__float_as_uint(Bs[SF_MASK_LO * n + seed])) |
+            (static_cast<unsigned long long>(__float_as_uint(Bs[SF_MASK_HI * n + seed])) << 32);
+        const int dir = __float_as_int(Bs[SF_DIR * n + seed]);
+        uint32_t status = tid == 0 ? __float_as_uint(Bs[SF_STATUS * n + seed]) : 0u;
+        // the fitted seed, or (step1) the seed after its first step: candidate r
+        // becomes its child r
+        float p[6], C[21];
+        Lo lo;
+        Innov I;
+#pragma unroll
+        for (int i = 0; i < 6; ++i) p[i] = Bs[(SF_P + i) * n + seed];
+        lo.x = Bs[(SF_LO + 0) * n + seed];
+        lo.y = Bs[(SF_LO + 1) * n + seed];
+        lo.z = Bs[(SF_LO + 2) * n + seed];
+        lo.phi = Bs[(SF_LO + 3) * n + seed];
+        lo.th = Bs[SF_LOTH * n + seed];
+#pragma unroll
+        for (int k = 0; k < 21; ++k) C[k] = Bs[(SF_C + k) * n + seed];
+#pragma unroll
+        for (int k = 0; k < 6; ++k) I.HCu[k] = I.HCv[k] = 0.f;
+        I.Suu = I.Suv = I.Svv = I.Iuu = I.Iuv = I.Ivv = 0.f;
+        float chi2 = Bs[SF_CHI2 * n + seed];
+        Book bk = unpack_book(__float_as_uint(Bs[SF_BOOK * n + seed]));
+        int c_cl = 0, c_ht = 0, c_up = 0, step = 0;
+        bool live = lane_used && rank == 0, pend = false;
+        uint32_t pcode = 0;
+        float pu = 0.f, pv = 0.f, px2 = 0.f;
+        if (A.step1) {
+            const int nb = __float_as_int(Bs[SF_BEAM * n + seed]), nl = __float_as_int(Bs[SF_NLIST * n + seed]);
+            if (tid == 0) {
+                c_cl = __float_as_int(Bs[SF_CCL * n + seed]);
+                c_ht = __float_as_int(Bs[SF_CHT * n + seed]);
+            }
+            live = lane_used && rank < nb;
+            pend = live;
+            pcode = __float_as_int(Bs[SF_SEARCHED * n + seed]) ? kCodeMiss : kCodePass;
+            if (live && rank < nl) {
+#pragma unroll
+                for (int k = 0; k < 6; ++k) {
+                    I.HCu[k] = Bs[(SF_I + k) * n + seed];
+                    I.HCv[k] = Bs[(SF_I + 6 + k) * n + seed];
+                }
+                I.Iuu = Bs[(SF_I + 12) * n + seed];
+                I.Iuv = Bs[(SF_I + 13) * n + seed];
+                I.Ivv = Bs[(SF_I + 14) * n + seed];
+                const float *L = A.beam;
+                px2 = L[((int64_t)rank * kListFields + LF_CHI2) * n + seed];
+                pcode = __float_as_uint(L[((int64_t)rank * kListFields + LF_ORIG) * n + seed]);
+                pu = L[((int64_t)rank * kListFields + LF_U) * n + seed];
+                pv = L[((int64_t)rank * kListFields + LF_V) * n + seed];
+            }
+            if (lead && live) hist[rank] = pcode;  // parent rank 0
+            step = 1;
+        }
+        while (true) {
+            if (pend) {
+                make_child(pcode, I, pu, pv, px2, A.max_consec, p, lo, C, chi2, bk, c_up);
+                pend = false;
+            }
+            if (step >= A.max_steps) {
+                if (tid == 0) record_fault(A.fault, kFaultHistOverflow, seed);
+                break;
+            }
+            const bool active = live && !bk.done;
+            if (!__syncthreads_or(active)) break;
+            Expansion X{-1, false, 0, 0, 0.f, false};
+            if (active)
+                expand<kPhys, false, true>(A, G, ev, mask, dir, N, cut, p, lo, C, bk, I, status, c_cl, c_ht,
+                                           lchi + tid, lorig + tid, lu + tid, lv + tid, nt, X, sub, lanes);
+            // the candidate's list from its lanes' lists: the smallest remaining
+            // (chi2, hit index) of the lanes' heads, N times
+            int head = 0, nlist = 0;
+            for (int j = 0; j < N; ++j) {
+                unsigned long long key = ~0ull;
+                if (head < X.nlist)
+                    // + 0: minus zero ranks as zero, as in the lists' comparisons
+                    key = (static_cast<unsigned long long>(ord_float(lchi[head * nt + tid] + 0.f)) << 32) |
+                          static_cast<uint32_t>(lorig[head * nt + tid]);
+                unsigned long long best = key;
+                for (int off = lanes >> 1; off > 0; off >>= 1) {
+                    const unsigned long long o = __shfl_xor_sync(kFull, best, off);
+                    best = o < best ? o : best;
+                }
+                if (!__any_sync(kFull, best != ~0ull)) break;
+                if (best != ~0ull) {
+                    ++nlist;
+                    if (key == best) {
+                        mchi[j * kWideRanks + row] = lchi[head * nt + tid];
+                        morig[j * kWideRanks + row] = lorig[head * nt + tid];
+                        mu[j * kWideRanks + row] = lu[head * nt + tid];
+                        mv[j * kWideRanks + row] = lv[head * nt + tid];
+                        ++head;
+                    }
+                }
+            }
+            __syncwarp();
+            if (kLearned) {  // the gate, N = 1 (the other learned calls leave no seeds here)
+                int compat = X.n_compat;
+                for (int off = lanes >> 1; off > 0; off >>= 1) compat += __shfl_xor_sync(kFull, compat, off);
+                if (X.searched && nlist > 0 && compat >= 2) {
+                    float fe[12];
+                    pair_features(mu[row], mv[row], I, mchi[row], cut, chi2, bk, X.layer, G.n_layers, G.L[X.layer].kind,
+                                  p, X.cot, fe);
+                    if (mlp_logit(WS, fe) < A.mlp_tau) status |= MKF_ST_AMBIG;
+                }
+            }
+            if (lead) {
+                float *S = state + rank * kWideState;
+#pragma unroll
+                for (int i = 0; i < 6; ++i) S[i] = p[i];
+                S[6] = lo.x;
+                S[7] = lo.y;
+                S[8] = lo.z;
+                S[9] = lo.phi;
+                S[10] = lo.th;
+#pragma unroll
+                for (int k = 0; k < 21; ++k) S[11 + k] = C[k];
+#pragma unroll
+                for (int k = 0; k < 6; ++k) {
+                    S[32 + k] = I.HCu[k];
+                    S[38 + k] = I.HCv[k];
+                }
+                S[44] = I.Iuu;
+                S[45] = I.Iuv;
+                S[46] = I.Ivv;
+                S[47] = chi2;
+                S[48] = __uint_as_float(pack_book(bk));
+                S[49] = __int_as_float(live ? (X.searched ? nlist + 1 : 1) : 0);
+                S[50] = __int_as_float(nlist);
+                S[51] = __int_as_float(X.searched ? 1 : 0);
+            }
+            __syncthreads();
+            // the N best children, as in find_kernel: lane r holds candidate r's keys
+            if (tid < 32) {
+                const int r = tid < N ? tid : 0;
+                const float *S = state + r * kWideState;
+                const int nl = __float_as_int(S[50]);
+                const int n_children = tid < N ? __float_as_int(S[49]) : 0;
+                const float score = cut * static_cast<float>(unpack_book(__float_as_uint(S[48])).nh) - S[47];
+                const uint32_t nohit = __float_as_int(S[51]) ? kCodeMiss : kCodePass;
+                const uint32_t tag = 15u - static_cast<uint32_t>(r);
+                int h = 0, got = 0;
+                for (int j = 0; j < N; ++j) {
+                    uint32_t key = 0u;
+                    if (h < n_children)
+                        key = sel_key(h < nl ? score + cut - mchi[h * kWideRanks + r] : score, tag);
+                    const uint32_t m = __reduce_max_sync(kFull, key);
+                    if (m == 0u) break;
+                    ++got;
+                    if (key == m) {  // keys are unique: one lane
+                        hist[step * kWideRanks + j] =
+                            (static_cast<uint32_t>(r) << 28) |
+                            (h < nl ? static_cast<uint32_t>(morig[h * kWideRanks + r]) : nohit);
+                        sel[j] = h;
+                        ++h;
+                    }
+                }
+                if (tid == 0) s_got = got;
+            }
+            __syncthreads();
+            // each candidate's lanes become its child
+            live = lane_used && rank < s_got;
+            if (live) {
+                const uint32_t rec = hist[step * kWideRanks + rank];
+                const int parent = static_cast<int>(rec >> 28);
+                const float *S = state + parent * kWideState;
+#pragma unroll
+                for (int i = 0; i < 6; ++i) p[i] = S[i];
+                lo.x = S[6];
+                lo.y = S[7];
+                lo.z = S[8];
+                lo.phi = S[9];
+                lo.th = S[10];
+#pragma unroll
+                for (int k = 0; k < 21; ++k) C[k] = S[11 + k];
+#pragma unroll
+                for (int k = 0; k < 6; ++k) {
+                    I.HCu[k] = S[32 + k];
+                    I.HCv[k] = S[38 + k];
+                }
+                I.Iuu = S[44];
+                I.Iuv = S[45];
+                I.Ivv = S[46];
+                chi2 = S[47];
+                bk = unpack_book(__float_as_uint(S[48]));
+                pcode = rec & kHitMask;
+                const bool hit = pcode < kCodeMiss;
+                const int at = (hit ? sel[rank] : 0) * kWideRanks + parent;
+                pu = hit ? mu[at] : 0.f;
+                pv = hit ? mv[at] : 0.f;
+                px2 = hit ? mchi[at] : 0.f;
+                pend = true;
+            }
+            ++step;
+            // the next write of these rows is behind the __syncthreads_or above
+        }
+        // output: candidate 0 is the best
+        if (lead) {
+            atomicAdd(&s_cl, c_cl);
+            atomicAdd(&s_up, c_up);
+        }
+        if (c_ht) atomicAdd(&s_ht, c_ht);
+        if (status) atomicOr(&s_status, status);
+        __syncthreads();
+        if (tid == 0) {
+            c_cl = s_cl;
+            c_ht = s_ht;
+            c_up = s_up;
+            status = s_status;
+            write_track(A, seed, ev, status, live, bk, p, lo, C, chi2, __float_as_int(Bs[(SF_HITS + 0) * n + seed]),
+                        __float_as_int(Bs[(SF_HITS + 1) * n + seed]), __float_as_int(Bs[(SF_HITS + 2) * n + seed]), hist,
+                        kWideRanks, 0, step, c_cl, c_ht, c_up);
+        }
+    }
+}
+
+}  // namespace
+
 extern "C" mkf_status mkf_find(mkf_ctx *ctx, const mkf_hitbins *bins, const int32_t *seed_hits,
                                const int32_t *seed_event, int32_t n_seeds, const mkf_find_params *params,
                                float *out_par, float *out_cov, float *chi2, int32_t *n_hits, int32_t *hit_idx,
@@ -1231,10 +1608,17 @@ extern "C" mkf_status mkf_find(mkf_ctx *ctx, const mkf_hitbins *bins, const int3
         reinterpret_cast<const void *>(find_kernel<true, 1, 10>), reinterpret_cast<const void *>(find_kernel<true, 2, 0>),
         reinterpret_cast<const void *>(find_kernel<true, 2, 0>), reinterpret_cast<const void *>(find_kernel<true, 2, 0>)};
     const void *kfn = kfns[vi];
+    const void *const wfns[3] = {reinterpret_cast<const void *>(find_wide_kernel<false, 1>),
+                                 reinterpret_cast<const void *>(find_wide_kernel<false, 2>),
+                                 reinterpret_cast<const void *>(find_wide_kernel<true, 1>)};
+    const void *wfn = wfns[learned ? 2 : (phys == 2 ? 1 : 0)];
     if (static_cast<int>(smem) > ctx->find_smem_attr) {
         const int want = static_cast<int>(std::max<size_t>(smem, 48 * 1024));
         for (int v = 0; v < 18; ++v)
             MKF_CUDA_TRY(cudaFuncSetAttribute(kfns[v], cudaFuncAttributeMaxDynamicSharedMemorySize, want));
+        for (const void *w : wfns)
+            MKF_CUDA_TRY(cudaFuncSetAttribute(w, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              static_cast<int>(wide_smem_bytes(MKF_MAX_LAYERS, MKF_MAX_NBEST))));
         ctx->find_smem_attr = want;
     }
     void *scratch = nullptr;
@@ -1248,11 +1632,21 @@ extern "C" mkf_status mkf_find(mkf_ctx *ctx, const mkf_hitbins *bins, const int3
     const int n_keys = bins->n_events * kOrderBuckets;
     const size_t order_bytes =
         grouped ? ((sizeof(int32_t) * (3 * (size_t)n_seeds + n_keys + 1) + 255) / 256) * 256 : 0;
-    mkf_status st = mkf_scratch(ctx, seed_bytes + beam_bytes + order_bytes + 256, &scratch);
+    // seeds with a wide window go to find_wide_kernel: with material, in the
+    // plain finder and in the cascade's best-hit pass
+    const bool leave = learned ? phys == 1 && params->mlp_mode == 1 && N == 1 : phys >= 1;
+    const size_t wide_bytes = leave ? ((sizeof(int32_t) * (size_t)n_seeds + 255) / 256) * 256 : 0;
+    mkf_status st = mkf_scratch(ctx, seed_bytes + beam_bytes + order_bytes + wide_bytes + 256, &scratch);
     if (st != MKF_OK) return st;
     A.seedbuf = static_cast<float *>(scratch);
     A.beam = A.step1 ? reinterpret_cast<float *>(static_cast<char *>(scratch) + seed_bytes) : nullptr;
-    A.work_counter = reinterpret_cast<int32_t *>(static_cast<char *>(scratch) + seed_bytes + beam_bytes + order_bytes);
+    char *const tail = static_cast<char *>(scratch) + seed_bytes + beam_bytes + order_bytes;
+    A.work_counter = reinterpret_cast<int32_t *>(tail + wide_bytes);
+    A.wide_list = leave ? reinterpret_cast<int32_t *>(tail) : nullptr;
+    A.wide_count = A.work_counter + 1;
+    A.wide_next = A.work_counter + 2;
+    const int64_t wide_bins = kWideHits * bins->n_bins / std::max(1, bins->n_hits);
+    A.wide_bins = static_cast<int32_t>(std::min<int64_t>(std::max<int64_t>(wide_bins, 1), 1 << 30));
     int32_t *order = nullptr;
     A.order_key = A.order_pos = A.order_counts = nullptr;
     if (grouped) {
@@ -1264,7 +1658,8 @@ extern "C" mkf_status mkf_find(mkf_ctx *ctx, const mkf_hitbins *bins, const int3
         MKF_CUDA_TRY(cudaMemsetAsync(A.order_counts, 0, sizeof(int32_t) * (n_keys + 1), ctx->stream));
     }
     A.event_times = reinterpret_cast<unsigned long long *>(params->event_times);
-    MKF_CUDA_TRY(cudaMemsetAsync(A.work_counter, 0, sizeof(int32_t), ctx->stream));
+    // the list of seeds left and the counters behind it
+    MKF_CUDA_TRY(cudaMemsetAsync(tail, 0, wide_bytes + 3 * sizeof(int32_t), ctx->stream));
     if (A.event_times) {
         MKF_CUDA_TRY(cudaMemsetAsync(A.event_times, 0, sizeof(uint64_t) * bins->n_events, ctx->stream));
         MKF_CUDA_TRY(cudaMemsetAsync(A.event_times + bins->n_events, 0xff, sizeof(uint64_t), ctx->stream));
@@ -1303,6 +1698,22 @@ extern "C" mkf_status mkf_find(mkf_ctx *ctx, const mkf_hitbins *bins, const int3
     const int blocks = std::max(1, std::min(need, std::max(1, per_sm) * ctx->num_sms));
     void *kargs[1] = {&A};
     MKF_CUDA_TRY(cudaLaunchKernel(kfn, dim3(blocks), dim3(threads), kargs, smem, ctx->stream));
+    if (leave) {
+        // how many seeds were left is known on the device only: the blocks that
+        // find none exit at once
+        const int wide_blocks = std::min(n_seeds, 3 * ctx->num_sms);
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(wide_blocks);
+        cfg.blockDim = dim3(wide_threads(N));
+        cfg.dynamicSmemBytes = wide_smem_bytes(ctx->geom.n_layers, N);
+        cfg.stream = ctx->stream;
+        cudaLaunchAttribute attr = {};
+        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr.val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        MKF_CUDA_TRY(cudaLaunchKernelExC(&cfg, wfn, kargs));
+    }
     return MKF_OK;
 }
 
