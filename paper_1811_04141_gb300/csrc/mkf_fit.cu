@@ -99,17 +99,125 @@ __device__ __forceinline__ bool update_with(const LayerDesc &Ld, float xh, float
     return true;
 }
 
+// One row of a track's hit list: the hit (-1: none) with its layer and position.
+struct HitRow {
+    int h, l;
+    float x, y, z;
+};
+
+// A track's hits row by row (kBackward: from the last row), each copied into
+// shared memory while the row before it is processed, its index loaded one row
+// earlier still: the gathers (four of them behind an index load, 700 cycles
+// each from L2) then cost the filter no wait.  Every thread waits for its own
+// copies only.  An index outside [0, n_hits) is a device fault and taken as no hit.
+constexpr int kFitThreads = 128;
+
+template <bool kBackward>
+struct HitFeed {
+    const FitArgs &A;
+    const int t;
+    int kk = 0;       // rows handed out
+    int h0, h1 = -1;  // the next row's hit (its copy is under way) and the one after
+    __device__ __forceinline__ int row(int i) const { return kBackward ? A.max_hits - 1 - i : i; }
+    __device__ __forceinline__ int index(int i) const {
+        return i < A.max_hits ? A.hit_idx[(int64_t)row(i) * A.n + t] : -1;
+    }
+    __device__ __forceinline__ int checked(int h) const {
+        if (h < A.n_hits) return h < 0 ? -1 : h;
+        record_fault(A.fault, kFaultBadHitIndex, t);
+        return -1;
+    }
+#ifdef __CUDACC__
+    float (*buf)[4][kFitThreads];
+    __device__ __forceinline__ void copy(int i, int h) {
+        if (h >= 0) {
+            const void *src[4] = {A.X + h, A.Y + h, A.Z + h, A.hit_layer + h};
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const unsigned dst = static_cast<unsigned>(__cvta_generic_to_shared(&buf[i & 1][c][threadIdx.x]));
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(dst), "l"(src[c]));
+            }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    __device__ __forceinline__ HitFeed(const FitArgs &A_, int t_, float (*buf_)[4][kFitThreads])
+        : A(A_), t(t_), buf(buf_) {
+        h0 = checked(index(0));
+        h1 = index(1);
+        copy(0, h0);
+    }
+    // the next row; false after the last one
+    __device__ __forceinline__ bool next(HitRow &r) {
+        if (kk >= A.max_hits) return false;
+        r.h = h0;
+        h0 = checked(h1);
+        copy(kk + 1, h0);
+        h1 = index(kk + 2);
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        const float (*b)[kFitThreads] = buf[kk & 1];
+        if (r.h >= 0) {
+            r.x = b[0][threadIdx.x];
+            r.y = b[1][threadIdx.x];
+            r.z = b[2][threadIdx.x];
+            r.l = __float_as_int(b[3][threadIdx.x]);
+        }
+        ++kk;
+        return true;
+    }
+#else
+    HitFeed(const FitArgs &A_, int t_, float (*)[4][kFitThreads]) : A(A_), t(t_) {}
+    bool next(HitRow &r) {
+        if (kk >= A.max_hits) return false;
+        r.h = checked(index(kk++));
+        if (r.h >= 0) {
+            r.x = A.X[r.h];
+            r.y = A.Y[r.h];
+            r.z = A.Z[r.h];
+            r.l = A.hit_layer[r.h];
+        }
+        return true;
+    }
+#endif
+    // the row handed out last
+    __device__ __forceinline__ int k() const { return row(kk - 1); }
+};
+
+// The first three hits of a track's list (false: it has fewer); reports the
+// invalid indices on the way.
+__device__ __forceinline__ bool first_three(const FitArgs &A, int t, int first[3]) {
+    int nfirst = 0;
+    // the first three rows at once: nearly always the three hits
+    int h[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) h[k] = k < A.max_hits ? A.hit_idx[(int64_t)k * A.n + t] : -1;
+    for (int k = 0; k < A.max_hits && nfirst < 3; ++k) {
+        const int hk = k == 0 ? h[0] : k == 1 ? h[1] : k == 2 ? h[2] : A.hit_idx[(int64_t)k * A.n + t];
+        if (hk >= A.n_hits) record_fault(A.fault, kFaultBadHitIndex, t);
+        if (hk < 0 || hk >= A.n_hits) continue;
+        if (nfirst == 0) first[0] = hk;
+        else if (nfirst == 1) first[1] = hk;
+        else first[2] = hk;
+        ++nfirst;
+    }
+    return nfirst >= 3;
+}
+
 // kBackward: hits in reverse order from the given state at the last hit, turned
 // around and inflated; the result at the first hit is turned back.  kPhys: 0
 // uniform field without material; 1 material effects compiled in (selected
 // when any layer has material); 2 the parameterised field (Runge-Kutta
 // propagation) with the material effects.
 template <bool kBackward, int kPhys>
-__global__ void __launch_bounds__(128, kPhys == 2 ? 4 : 6) fit_kernel(const __grid_constant__ FitArgs A) {
+__global__ void __launch_bounds__(128, kPhys == 0 ? 5 : 4) fit_kernel(const __grid_constant__ FitArgs A) {
     constexpr bool kMaterial = kPhys >= 1, kParamField = kPhys == 2;
     constexpr int kSq = kMaterial ? 9 : 5;  // square-root columns through the seed hits
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= A.n) return;
+#ifdef __CUDACC__
+    __shared__ float buf[2][4][kFitThreads];
+#else
+    float (*const buf)[4][kFitThreads] = nullptr;
+#endif
     const Geom &G = A.G;
     float p[6], C[21];
     SqrtCov<kSq> Q;
@@ -118,18 +226,8 @@ __global__ void __launch_bounds__(128, kPhys == 2 ? 4 : 6) fit_kernel(const __gr
     float chi2 = 0.f;
     int used = 0;
 
-    // first three valid hits (seed) and validity of all indices
-    int first[3] = {-1, -1, -1}, nfirst = 0;
-    for (int k = 0; k < A.max_hits; ++k) {
-        int h = A.hit_idx[(int64_t)k * A.n + t];
-        if (h < 0) continue;
-        if (h >= A.n_hits) {
-            record_fault(A.fault, kFaultBadHitIndex, t);
-            continue;
-        }
-        if (nfirst < 3) first[nfirst++] = h;
-    }
-    bool ok = nfirst >= 3;
+    int first[3] = {-1, -1, -1};
+    bool ok = first_three(A, t, first);
     if (ok) {
         int l0 = A.hit_layer[first[0]];
         if (l0 < 0 || l0 >= G.n_layers) {
@@ -155,19 +253,23 @@ __global__ void __launch_bounds__(128, kPhys == 2 ? 4 : 6) fit_kernel(const __gr
             ok = seed_state(G.L[l0], kbs, h1, h2, h3, p, Q, eta);
         }
     }
-    if (!ok) st |= MKF_ST_BADSEED;
+    if (!ok) {
+        st |= MKF_ST_BADSEED;
+        // the list's invalid indices are reported all the same
+        for (int k = 0; k < A.max_hits; ++k)
+            if (A.hit_idx[(int64_t)k * A.n + t] >= A.n_hits) record_fault(A.fault, kFaultBadHitIndex, t);
+    }
 
     if (ok) {
         bool firsthit = true;
         // one hit: onto its layer (after the first), material, update; Cx is
         // the covariance (float[21]) or, through the seed hits, its square root
-        auto hit = [&](auto Cx, int h) {
-            const int l = A.hit_layer[h];
-            if (l < 0 || l >= G.n_layers) {
-                record_fault(A.fault, kFaultBadLayer, h);
+        auto hit = [&](auto Cx, const HitRow &r) {
+            if (r.l < 0 || r.l >= G.n_layers) {
+                record_fault(A.fault, kFaultBadLayer, r.h);
                 return;
             }
-            const LayerDesc &Ld = G.L[l];
+            const LayerDesc &Ld = G.L[r.l];
             if (!firsthit) {
                 if (!move_to<kPhys>(G, Ld, p, lo, Cx)) {
                     st |= MKF_ST_UNREACHABLE;
@@ -182,7 +284,7 @@ __global__ void __launch_bounds__(128, kPhys == 2 ? 4 : 6) fit_kernel(const __gr
             }
             firsthit = false;
             float dchi2;
-            if (update_with(Ld, A.X[h], A.Y[h], A.Z[h], p, lo, Cx, dchi2)) {
+            if (update_with(Ld, r.x, r.y, r.z, p, lo, Cx, dchi2)) {
                 chi2 += dchi2;
                 ++used;
             } else {
@@ -198,25 +300,17 @@ __global__ void __launch_bounds__(128, kPhys == 2 ? 4 : 6) fit_kernel(const __gr
                 add_scattering(Ld.kind, mx0, p, Cx);
             }
         };
-        auto hit_at = [&](int kk) {
-            const int k = kBackward ? A.max_hits - 1 - kk : kk;
-            const int h = A.hit_idx[(int64_t)k * A.n + t];
-            return h < 0 || h >= A.n_hits ? -1 : h;
-        };
-        int kk = 0;
+        HitFeed<kBackward> feed(A, t, buf);
+        HitRow r;
         if constexpr (!kBackward) {
             if (!A.seed_par) {  // from the seed prior: the seed hits with the square root
-                for (; kk < A.max_hits && used < 3; ++kk) {
-                    const int h = hit_at(kk);
-                    if (h >= 0) hit(&Q, h);
-                }
+                while (used < 3 && feed.next(r))
+                    if (r.h >= 0) hit(&Q, r);
                 sqrt_to_cov(Q, C);
             }
         }
-        for (; kk < A.max_hits; ++kk) {
-            const int h = hit_at(kk);
-            if (h >= 0) hit(C, h);
-        }
+        while (feed.next(r))
+            if (r.h >= 0) hit(C, r);
         if (kBackward) reverse_state(p, lo, C);
         if (!finite_state(p) || !isfinite(chi2)) st |= MKF_ST_NONFINITE;
     }
@@ -695,7 +789,7 @@ static mkf_status launch_fit(mkf_ctx *ctx, const float *xyz, const int32_t *hit_
     A.ndf = ndf;
     A.status = status;
     A.fault = ctx->fault;
-    const int threads = 128;
+    const int threads = kFitThreads;
     const int blocks = (n + threads - 1) / threads;
     if (mode == 2) {
         switch (mkf_phys_variant(ctx->geom)) {

@@ -83,6 +83,15 @@ __device__ __forceinline__ float wrap_pi(float a) {
     return a;
 }
 
+// a + b that the compiler does not merge with a product into an FMA.
+__device__ __forceinline__ float add_rn(float a, float b) {
+#ifdef __CUDA_ARCH__
+    return __fadd_rn(a, b);
+#else
+    return a + b;
+#endif
+}
+
 // Error-free transformations (Knuth two-sum, FMA two-product).
 __device__ __forceinline__ void two_sum(float a, float b, float &s, float &e) {
     s = a + b;
@@ -99,6 +108,18 @@ __device__ __forceinline__ void two_prod(float a, float b, float &p, float &e) {
 __device__ __forceinline__ void df_add(float &hi, float &lo, float d) {
     float s, e;
     two_sum(hi, d, s, e);
+    e += lo;
+    hi = s + e;
+    lo = e - (hi - s);
+}
+
+// (hi, lo) += m * n
+template <bool kF1, bool kF2>
+__device__ __forceinline__ void df_add_prod(float &hi, float &lo, float m, float n) {
+    const float b = m * n;
+    const float s = kF1 ? fmaf(m, n, hi) : add_rn(hi, b);
+    const float bb = add_rn(s, -hi);
+    float e = add_rn(add_rn(hi, -add_rn(s, -bb)), kF2 ? fmaf(m, n, -bb) : add_rn(b, -bb));
     e += lo;
     hi = s + e;
     lo = e - (hi - s);
@@ -376,13 +397,13 @@ __device__ __forceinline__ void propagate_transport(const LayerDesc& Ld, float k
     sincos_small(a, sa, ca);
     sinc_and_deriv(a, sa, ca, sn, dsn);
     const float L = s * sn;
-    const float cm = cphi * ca - sphi * sa, sm = sphi * ca + cphi * sa;  // direction phi + a
+    const float cm = fmaf(cphi, ca, -(sphi * sa)), sm = fmaf(sphi, ca, cphi * sa);  // direction phi + a
     const float dx = L * cm, dy = L * sm;
     const float c2a = 1.f - 2.f * sa * sa, s2a = 2.f * sa * ca;
-    const float cpe = cphi * c2a - sphi * s2a, spe = sphi * c2a + cphi * s2a;  // direction at the end
+    const float cpe = fmaf(cphi, c2a, -(sphi * s2a)), spe = fmaf(cphi, s2a, sphi * c2a);  // direction at the end
     float st, ct_unused;
     sincos_small(p[5], st, ct_unused);
-    const float xe = p[0] + dx, ye = p[1] + dy;
+    const float xe = add_rn(p[0], dx), ye = add_rn(p[1], dy);
 
     HelixJac J;
     J.kind = Ld.kind;
@@ -415,13 +436,13 @@ __device__ __forceinline__ void propagate_transport(const LayerDesc& Ld, float k
     }
     transport_cov(J, C);
 
-    df_add(p[0], lo.x, dx);
-    df_add(p[1], lo.y, dy);
+    df_add_prod<false, false>(p[0], lo.x, L, cm);
+    df_add_prod<false, false>(p[1], lo.y, L, sm);
     if (Ld.kind == 1) {
         p[2] = Ld.rz;  // on the disk by construction
         lo.z = 0.f;
     } else {
-        df_add(p[2], lo.z, s * cot);
+        df_add_prod<true, true>(p[2], lo.z, s, cot);
     }
     df_add(p[4], lo.phi, 2.f * a);
     df_wrap_pi(p[4], lo.phi);
@@ -784,7 +805,7 @@ __device__ __forceinline__ bool scatter_angle(int kind, float t, const float p[6
     const float pm = 1.f / (fabsf(p[3]) * st);
     const float beta = pm / sqrtf(fmaf(pm, pm, kPionMass2));
     const float x = t / cosa;
-    th0 = 0.0136f / (beta * pm) * sqrtf(x) * (1.f + 0.038f * logf(x / (beta * beta)));
+    th0 = 0.0136f / (beta * pm) * sqrtf(x) * fmaf(0.038f, logf(x / (beta * beta)), 1.f);
     wc = p[3] * ct / st;
     return true;
 }
@@ -793,10 +814,10 @@ __device__ __forceinline__ void add_scattering(int kind, float t, const float p[
     float th0, wc, st;
     if (!scatter_angle(kind, t, p, th0, wc, st)) return;
     const float v = th0 * th0;
-    C[sym(5, 5)] += v;
-    C[sym(4, 4)] += v / (st * st);
-    C[sym(3, 3)] += wc * wc * v;
-    C[sym(5, 3)] -= wc * v;
+    C[sym(5, 5)] = add_rn(C[sym(5, 5)], v);
+    C[sym(4, 4)] = fmaf(v, 1.f / (st * st), C[sym(4, 4)]);
+    C[sym(3, 3)] = fmaf(wc * wc, v, C[sym(3, 3)]);
+    C[sym(5, 3)] = fmaf(-wc, v, C[sym(5, 3)]);
 }
 
 // The same noise as two columns of the square root: theta0 (-wc e_q/pT + e_theta)
@@ -846,13 +867,13 @@ __device__ __forceinline__ bool eloss_map(int kind, float t, float k, float p[6]
     const float e = sqrtf(fmaf(pm, pm, kPionMass * kPionMass));
     const float beta = pm / e;
     const float kx = sign * k * (t / cosa);
-    const float e2 = e - kx / (beta * beta);
+    const float e2 = fmaf(-kx, 1.f / (beta * beta), e);
     if (!(e2 > kPionMass)) return false;  // stopped: left as it is
     const float p2 = sqrtf(fmaf(e2, e2, -kPionMass * kPionMass));
     const float r = pm / p2;
-    const float dp2 = e2 / p2 * (pm / e + 2.f * kx * (kPionMass * kPionMass) / (pm * pm * pm));
-    const float gp = 1.f / p2 - pm * dp2 / (p2 * p2);
-    a = r - pm * gp;
+    const float dp2 = e2 / p2 * fmaf(2.f * kx * (kPionMass * kPionMass), 1.f / (pm * pm * pm), pm / e);
+    const float gp = fmaf(-(pm * dp2), 1.f / (p2 * p2), 1.f / p2);
+    a = fmaf(-pm, gp, r);
     c = -p[3] * pm * (ct / st) * gp;
     p[3] *= r;
     return true;
@@ -1053,7 +1074,7 @@ __device__ __forceinline__ float sqrt_update(int kind, float su2, float sv2, con
 #pragma unroll
     for (int j = 0; j < K; ++j) ph[j] = fmaf(-f.sp, Q->S[0][j], f.cp * Q->S[1][j]);
     float chi2 = potter_step(Q->S, ph, su2, u, dp);
-    const float v2 = v - (kind == 0 ? dp[2] : fmaf(f.cp, dp[0], f.sp * dp[1]));
+    const float v2 = add_rn(v, -(kind == 0 ? dp[2] : fmaf(f.cp, dp[0], f.sp * dp[1])));
 #pragma unroll
     for (int j = 0; j < K; ++j) ph[j] = kind == 0 ? Q->S[2][j] : fmaf(f.cp, Q->S[0][j], f.sp * Q->S[1][j]);
     chi2 += potter_step(Q->S, ph, sv2, v2, dp);
@@ -1100,7 +1121,7 @@ __device__ __forceinline__ bool seed_state(const LayerDesc& L1, float kb, const 
     if (kb != 0.f) w = -h / kb;
     else h = 0.f;
     float xa = 0.5f * h * la, xb = 0.5f * h * lb;
-    float phi0 = atan2f(ay, ax) - xa * asinc(xa);
+    float phi0 = fmaf(-xa, asinc(xa), atan2f(ay, ax));
     float s13 = lb * asinc(xb);
     float cot = (h3[2] - h1[2]) / s13;
     p[0] = h1[0];
