@@ -348,8 +348,19 @@ __global__ void __launch_bounds__(128, kPhys == 0 ? 5 : 4) fit_kernel(const __gr
 __device__ __forceinline__ bool combine5(int kind, float rz, const float pf_[6], const float Cf_[21],
                                          const float pb_[6], const float Cb_[21], float ps[6], float Cs[21]) {
     const bool swap = Cb_[9] < Cf_[9];
-    const float *pf = swap ? pb_ : pf_, *Cf = swap ? Cb_ : Cf_;  // base
-    const float *pb = swap ? pf_ : pb_, *Cb = swap ? Cf_ : Cb_;  // other
+    // base (pf, Cf) and other (pb, Cb), by selects: a pointer that chooses
+    // between two arrays would put both in local memory
+    float pf[6], pb[6], Cf[21], Cb[21];
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+        pf[i] = swap ? pb_[i] : pf_[i];
+        pb[i] = swap ? pf_[i] : pb_[i];
+    }
+#pragma unroll
+    for (int i = 0; i < 21; ++i) {
+        Cf[i] = swap ? Cb_[i] : Cf_[i];
+        Cb[i] = swap ? Cf_[i] : Cb_[i];
+    }
     float c = 1.f, sn = 0.f;
     if (kind == 0) {
         const float ir = 1.f / sqrtf(fmaf(pf[0], pf[0], pf[1] * pf[1]));
@@ -577,19 +588,24 @@ __device__ __forceinline__ bool combine5(int kind, float rz, const float pf_[6],
 // (combine5) and is updated with the hit, its material applied in reverse.  The
 // last hit's row keeps the forward state.
 template <int kPhys>
-__global__ void __launch_bounds__(128, 4) smooth_kernel(const __grid_constant__ FitArgs A) {
+__global__ void __launch_bounds__(128, 3) smooth_kernel(const __grid_constant__ FitArgs A) {
     constexpr bool kMaterial = kPhys >= 1, kParamField = kPhys == 2;
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= A.n) return;
     const Geom &G = A.G;
     const float nanv = __int_as_float(0x7fc00000);
     const int64_t n = A.n;
-    for (int k = 0; k < A.max_hits; ++k) {
+#ifdef __CUDACC__
+    __shared__ float buf[2][4][kFitThreads];
+#else
+    float (*const buf)[4][kFitThreads] = nullptr;
+#endif
+    auto no_state = [&](int k) {
 #pragma unroll
         for (int i = 0; i < 6; ++i) A.sm_par[((int64_t)k * 6 + i) * n + t] = nanv;
 #pragma unroll
         for (int i = 0; i < 21; ++i) A.sm_cov[((int64_t)k * 21 + i) * n + t] = nanv;
-    }
+    };
     constexpr int kSq = kMaterial ? 9 : 5;  // square-root columns through the seed hits
     float p[6], C[21];
     SqrtCov<kSq> Q;
@@ -597,17 +613,8 @@ __global__ void __launch_bounds__(128, 4) smooth_kernel(const __grid_constant__ 
     uint32_t st = 0;
     float chi2 = 0.f;
     int used = 0;
-    int first[3] = {-1, -1, -1}, nfirst = 0;
-    for (int k = 0; k < A.max_hits; ++k) {
-        const int h = A.hit_idx[(int64_t)k * n + t];
-        if (h < 0) continue;
-        if (h >= A.n_hits) {
-            record_fault(A.fault, kFaultBadHitIndex, t);
-            continue;
-        }
-        if (nfirst < 3) first[nfirst++] = h;
-    }
-    bool ok = nfirst >= 3;
+    int first[3] = {-1, -1, -1};
+    bool ok = first_three(A, t, first);
     if (ok) {
         const int l0 = A.hit_layer[first[0]];
         if (l0 < 0 || l0 >= G.n_layers) {
@@ -627,21 +634,30 @@ __global__ void __launch_bounds__(128, 4) smooth_kernel(const __grid_constant__ 
             ok = seed_state(G.L[l0], kbs, h1, h2, h3, p, Q, eta);
         }
     }
-    if (!ok) st |= MKF_ST_BADSEED;
+    if (!ok) {
+        st |= MKF_ST_BADSEED;
+        // no states; the list's invalid indices are reported all the same
+        for (int k = 0; k < A.max_hits; ++k) {
+            if (A.hit_idx[(int64_t)k * n + t] >= A.n_hits) record_fault(A.fault, kFaultBadHitIndex, t);
+            no_state(k);
+        }
+    }
 
-    // forward filter, its state after each hit kept in the hit's row
+    // forward filter, its state after each hit kept in the hit's row (every row
+    // is written once here: with all rows set to NaN first, a pass more over the
+    // output, the smoother took 332 us for 10^5 tracks of 12 rows)
     int lastk = -1;
+    unsigned long long have = 0;  // rows with a forward state
     if (ok) {
         bool firsthit = true;
         // one hit; Cx is the covariance (float[21]) or, through the seed hits,
         // its square root
-        auto fwd = [&](auto Cx, int k, int h) {
-            const int l = A.hit_layer[h];
-            if (l < 0 || l >= G.n_layers) {
-                record_fault(A.fault, kFaultBadLayer, h);
+        auto fwd = [&](auto Cx, int k, const HitRow &r) {
+            if (r.l < 0 || r.l >= G.n_layers) {
+                record_fault(A.fault, kFaultBadLayer, r.h);
                 return;
             }
-            const LayerDesc &Ld = G.L[l];
+            const LayerDesc &Ld = G.L[r.l];
             if (!firsthit) {
                 if (!move_to<kPhys>(G, Ld, p, lo, Cx)) {
                     st |= MKF_ST_UNREACHABLE;
@@ -656,7 +672,7 @@ __global__ void __launch_bounds__(128, 4) smooth_kernel(const __grid_constant__ 
             }
             firsthit = false;
             float dchi2;
-            if (update_with(Ld, A.X[h], A.Y[h], A.Z[h], p, lo, Cx, dchi2)) {
+            if (update_with(Ld, r.x, r.y, r.z, p, lo, Cx, dchi2)) {
                 chi2 += dchi2;
                 ++used;
                 const float pw[6] = {p[0] + lo.x, p[1] + lo.y, p[2] + lo.z, p[3], p[4] + lo.phi, p[5] + lo.th};
@@ -672,22 +688,23 @@ __global__ void __launch_bounds__(128, 4) smooth_kernel(const __grid_constant__ 
 #pragma unroll
                 for (int i = 0; i < 21; ++i) A.sm_cov[((int64_t)k * 21 + i) * n + t] = Cw[i];
                 lastk = k;
+                have |= 1ull << k;
             } else {
                 st |= MKF_ST_BADS;
             }
         };
-        int k = 0;
+        HitFeed<false> feed(A, t, buf);
+        HitRow r;
+        auto row = [&](auto Cx) {
+            const int k = feed.k();
+            if (r.h >= 0) fwd(Cx, k, r);
+            if (!((have >> k) & 1ull)) no_state(k);
+        };
         if (!A.seed_par) {  // from the seed prior: the seed hits with the square root
-            for (; k < A.max_hits && used < 3; ++k) {
-                const int h = A.hit_idx[(int64_t)k * n + t];
-                if (h >= 0 && h < A.n_hits) fwd(&Q, k, h);
-            }
+            while (used < 3 && feed.next(r)) row(&Q);
             sqrt_to_cov(Q, C);
         }
-        for (; k < A.max_hits; ++k) {
-            const int h = A.hit_idx[(int64_t)k * n + t];
-            if (h >= 0 && h < A.n_hits) fwd(C, k, h);
-        }
+        while (feed.next(r)) row(C);
     }
 
     // backward filter and the weighted means
@@ -709,8 +726,16 @@ __global__ void __launch_bounds__(128, 4) smooth_kernel(const __grid_constant__ 
                     st |= MKF_ST_UNREACHABLE;
                     continue;
                 }
-                const float c0 = A.sm_cov[((int64_t)k * 21) * n + t];
-                if (c0 == c0) {  // the forward filter has a state here
+                float pf[6], Cf[21];
+                bool had = (have >> k) & 1ull;  // the forward filter has a state here
+                if (had) {
+#pragma unroll
+                    for (int i = 0; i < 6; ++i) pf[i] = A.sm_par[((int64_t)k * 6 + i) * n + t];
+#pragma unroll
+                    for (int i = 0; i < 21; ++i) Cf[i] = A.sm_cov[((int64_t)k * 21 + i) * n + t];
+                    had = Cf[0] == Cf[0];
+                }
+                if (had) {
                     float pb[6] = {p[0] + lo.x, p[1] + lo.y, p[2] + lo.z, p[3], p[4], p[5]}, Cb[21];
                     Lo lb{0.f, 0.f, 0.f, lo.phi, lo.th};
 #pragma unroll
@@ -718,11 +743,7 @@ __global__ void __launch_bounds__(128, 4) smooth_kernel(const __grid_constant__ 
                     reverse_state(pb, lb, Cb);
                     pb[4] += lb.phi;
                     pb[5] += lb.th;
-                    float pf[6], Cf[21], ps[6], Cs[21];
-#pragma unroll
-                    for (int i = 0; i < 6; ++i) pf[i] = A.sm_par[((int64_t)k * 6 + i) * n + t];
-#pragma unroll
-                    for (int i = 0; i < 21; ++i) Cf[i] = A.sm_cov[((int64_t)k * 21 + i) * n + t];
+                    float ps[6], Cs[21];
                     const bool good = combine5(Ld.kind, Ld.rz, pf, Cf, pb, Cb, ps, Cs);
                     if (!good) st |= MKF_ST_BADS;
 #pragma unroll
