@@ -108,8 +108,11 @@ struct HitRow {
 // A track's hits row by row (kBackward: from the last row), each copied into
 // shared memory while the row before it is processed, its index loaded one row
 // earlier still: the gathers (four of them behind an index load, 700 cycles
-// each from L2) then cost the filter no wait.  Every thread waits for its own
-// copies only.  An index outside [0, n_hits) is a device fault and taken as no hit.
+// each from L2) then cost the filter no wait, and no registers (prefetched into
+// registers they spilled and gained nothing).  The kernel of one event of 1000
+// tracks went from 20.5 to 17.3 us; for 10^6 tracks see fit_kernel.  Every
+// thread waits for its own copies only.  An index outside [0, n_hits) is a device
+// fault and taken as no hit.
 constexpr int kFitThreads = 128;
 
 template <bool kBackward>
@@ -207,8 +210,15 @@ __device__ __forceinline__ bool first_three(const FitArgs &A, int t, int first[3
 // uniform field without material; 1 material effects compiled in (selected
 // when any layer has material); 2 the parameterised field (Runge-Kutta
 // propagation) with the material effects.
+// Bound: issue and instruction fetch (the uniform-field fit: 66 % of issue slots,
+// the hit code is there twice).  Blocks per SM, measured with the row feed:
+// uniform field 6 / 5 / 4: 334 / 322 / 333 us for 10^6 tracks of 10 hits (at 5
+// nothing spills; 336 us before the feed, at 6); material, out and back, 6 / 5 /
+// 4 / 3: 384 / 332 / 311 / 342 us for 144 000 tracks of 16 hits (367 us before,
+// at 6, where the square root of nine columns spilled 420 bytes a thread);
+// parameterised field 4 / 3 / 2: 547 / 497 / 512 us for 10^5 tracks of 10 hits.
 template <bool kBackward, int kPhys>
-__global__ void __launch_bounds__(128, kPhys == 0 ? 5 : 4) fit_kernel(const __grid_constant__ FitArgs A) {
+__global__ void __launch_bounds__(128, kPhys == 0 ? 5 : kPhys == 1 ? 4 : 3) fit_kernel(const __grid_constant__ FitArgs A) {
     constexpr bool kMaterial = kPhys >= 1, kParamField = kPhys == 2;
     constexpr int kSq = kMaterial ? 9 : 5;  // square-root columns through the seed hits
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
@@ -587,6 +597,10 @@ __device__ __forceinline__ bool combine5(int kind, float rz, const float pf_[6],
 // hit from the later ones, replaces the row by the weighted mean of the two
 // (combine5) and is updated with the hit, its material applied in reverse.  The
 // last hit's row keeps the forward state.
+// Bound: issue and the local memory of what does not fit in registers.  Blocks
+// per SM 5 / 4 / 3 / 2: 602 / 273 / 211 / 229 us for 10^5 tracks of 9 hits (12
+// rows); 334 us with every row set to NaN first, the two estimates of the mean
+// chosen through pointers (both then lay in local memory) and 4 blocks.
 template <int kPhys>
 __global__ void __launch_bounds__(128, 3) smooth_kernel(const __grid_constant__ FitArgs A) {
     constexpr bool kMaterial = kPhys >= 1, kParamField = kPhys == 2;
@@ -643,9 +657,8 @@ __global__ void __launch_bounds__(128, 3) smooth_kernel(const __grid_constant__ 
         }
     }
 
-    // forward filter, its state after each hit kept in the hit's row (every row
-    // is written once here: with all rows set to NaN first, a pass more over the
-    // output, the smoother took 332 us for 10^5 tracks of 12 rows)
+    // forward filter, its state after each hit kept in the hit's row (a row
+    // without one is set to NaN here, not all rows first: a pass less over the output)
     int lastk = -1;
     unsigned long long have = 0;  // rows with a forward state
     if (ok) {

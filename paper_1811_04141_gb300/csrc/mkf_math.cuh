@@ -30,6 +30,14 @@
 
 namespace mkf {
 
+// A function that is called, not inlined: where several copies of a long body
+// would crowd the instruction cache.
+#ifdef __CUDACC__
+#define MKF_CALLED static __device__ __noinline__
+#else
+#define MKF_CALLED static inline
+#endif
+
 constexpr float kPi = 3.14159265358979323846f;
 constexpr float kTwoPi = 6.28318530717958647692f;
 constexpr float kField = 0.0029979245800f;  // GeV / (T cm)
@@ -83,6 +91,9 @@ __device__ __forceinline__ float wrap_pi(float a) {
     return a;
 }
 
+// Where an expression leaves the compiler a choice of which product it merges
+// with a sum, the choice is written out below (fmaf, add_rn): left to it, two
+// kernels with the same source rounded differently.
 // a + b that the compiler does not merge with a product into an FMA.
 __device__ __forceinline__ float add_rn(float a, float b) {
 #ifdef __CUDA_ARCH__
@@ -113,13 +124,21 @@ __device__ __forceinline__ void df_add(float &hi, float &lo, float d) {
     lo = e - (hi - s);
 }
 
-// (hi, lo) += m * n
-template <bool kF1, bool kF2>
+// (hi, lo) += m n (merged into the sum and into its error term).
 __device__ __forceinline__ void df_add_prod(float &hi, float &lo, float m, float n) {
-    const float b = m * n;
-    const float s = kF1 ? fmaf(m, n, hi) : add_rn(hi, b);
+    const float s = fmaf(m, n, hi);
     const float bb = add_rn(s, -hi);
-    float e = add_rn(add_rn(hi, -add_rn(s, -bb)), kF2 ? fmaf(m, n, -bb) : add_rn(b, -bb));
+    float e = add_rn(add_rn(hi, -add_rn(s, -bb)), fmaf(m, n, -bb));
+    e += lo;
+    hi = s + e;
+    lo = e - (hi - s);
+}
+
+// (hi, lo) += d, d not merged with the product it may be.
+__device__ __forceinline__ void df_add_rn(float &hi, float &lo, float d) {
+    const float s = add_rn(hi, d);
+    const float bb = add_rn(s, -hi);
+    float e = add_rn(add_rn(hi, -add_rn(s, -bb)), add_rn(d, -bb));
     e += lo;
     hi = s + e;
     lo = e - (hi - s);
@@ -436,13 +455,13 @@ __device__ __forceinline__ void propagate_transport(const LayerDesc& Ld, float k
     }
     transport_cov(J, C);
 
-    df_add_prod<false, false>(p[0], lo.x, L, cm);
-    df_add_prod<false, false>(p[1], lo.y, L, sm);
+    df_add_rn(p[0], lo.x, dx);
+    df_add_rn(p[1], lo.y, dy);
     if (Ld.kind == 1) {
         p[2] = Ld.rz;  // on the disk by construction
         lo.z = 0.f;
     } else {
-        df_add_prod<true, true>(p[2], lo.z, s, cot);
+        df_add_prod(p[2], lo.z, s, cot);
     }
     df_add(p[4], lo.phi, 2.f * a);
     df_wrap_pi(p[4], lo.phi);
@@ -595,7 +614,7 @@ __device__ __forceinline__ void rk_step(float kb, float alpha, const float r0[3]
         T[i] = fmaf(h6 * lam, st[i] + S[3].tb[i], T[i]);
     }
     const float kba = kb * alpha;
-#pragma unroll
+#pragma unroll 1  // one column's code, see move_field
     for (int c = 0; c < 6; ++c) {
         float ar[3], at[3], ir[3], it[3], k[3];
         // stage 1
@@ -656,9 +675,15 @@ __device__ __forceinline__ float nearest_root(float a, float b, float c) {
 // parameter columns (dr, dT) integrated with the trajectory (the variational
 // equations, the field's gradient included), then the surface constraint
 // dS = -(n . dr) / (n . T) moves every column along (T, dT/dS) at the end.
-template <class Cov>
-__device__ __forceinline__ void propagate_field(const LayerDesc &Ld, float kb, float alpha, float p[6], Lo &lo,
-                                                Cov C, float sphi, float cphi, float h, float s) {
+// The code of this function is long, and fetching it was what bounded the
+// kernels in the field: the fit of 10^5 tracks of 10 hits took 866 us with two
+// copies of rk_step and six unrolled columns inlined for either covariance form,
+// 610 us with one copy of rk_step, 489 us with the columns in a loop as well
+// (their arrays then lie in local memory, which the first-level cache holds), 497
+// us as it is now, called instead of inlined (which keeps every bit of the
+// results, the inlined form did not).
+MKF_CALLED void move_field(const LayerDesc &Ld, float kb, float alpha, float p[6], Lo &lo,
+                                        float (&J)[6][6], float sphi, float cphi, float h, float s) {
     float st, ct;
     sincos_pair(p[5], lo.th, st, ct);
     const float lam = p[3] * st;
@@ -680,21 +705,23 @@ __device__ __forceinline__ void propagate_field(const LayerDesc &Ld, float kb, f
     const float nf = ceilf(fmaxf(fabsf(h) * s * (1.f / kRkTurn), fabsf(S) * (1.f / kRkLen)));
     const int n = nf >= 1.f ? (nf < static_cast<float>(kRkMaxN) ? static_cast<int>(nf) : kRkMaxN) : 1;
     const float hs = S / static_cast<float>(n);
-    for (int i = 0; i < n; ++i) rk_step(kb, alpha, r0, lam, dl, d, dlo, T, Dr, DT, hs);
-    for (int it = 0; it < kRkNewton; ++it) {
-        float dn;
-        if (Ld.kind == 0) {
-            // r^2 - R^2 from the position pair without cancellation
-            const float xl = (lo.x + dlo[0]) + d[0], yl = (lo.y + dlo[1]) + d[1];
-            const float x = p[0] + xl, y = p[1] + yl;
-            const float c = 2.f * fmaf(p[0], xl, p[1] * yl) + fmaf(xl, xl, yl * yl) - diff_sq2(Ld.rz, 0.f, p[0], p[1]);
-            float b[3];
-            kfield(kb, alpha, r0[0] + d[0], r0[1] + d[1], r0[2] + d[2], b);
-            const float Fx = lam * fmaf(T[1], b[2], -T[2] * b[1]), Fy = lam * fmaf(T[2], b[0], -T[0] * b[2]);
-            const float aq = fmaf(T[0], T[0], fmaf(T[1], T[1], fmaf(x, Fx, y * Fy)));
-            dn = nearest_root(aq, 2.f * fmaf(x, T[0], y * T[1]), c);
-        } else {
-            dn = ((Ld.rz - p[2]) - ((lo.z + dlo[2]) + d[2])) / T[2];
+    // one loop for the n steps and the corrections, so that rk_step is there once
+    for (int it = 0; it < n + kRkNewton; ++it) {
+        float dn = hs;
+        if (it >= n) {
+            if (Ld.kind == 0) {
+                // r^2 - R^2 from the position pair without cancellation
+                const float xl = (lo.x + dlo[0]) + d[0], yl = (lo.y + dlo[1]) + d[1];
+                const float x = p[0] + xl, y = p[1] + yl;
+                const float c = 2.f * fmaf(p[0], xl, p[1] * yl) + fmaf(xl, xl, yl * yl) - diff_sq2(Ld.rz, 0.f, p[0], p[1]);
+                float b[3];
+                kfield(kb, alpha, r0[0] + d[0], r0[1] + d[1], r0[2] + d[2], b);
+                const float Fx = lam * fmaf(T[1], b[2], -T[2] * b[1]), Fy = lam * fmaf(T[2], b[0], -T[0] * b[2]);
+                const float aq = fmaf(T[0], T[0], fmaf(T[1], T[1], fmaf(x, Fx, y * Fy)));
+                dn = nearest_root(aq, 2.f * fmaf(x, T[0], y * T[1]), c);
+            } else {
+                dn = ((Ld.rz - p[2]) - ((lo.z + dlo[2]) + d[2])) / T[2];
+            }
         }
         rk_step(kb, alpha, r0, lam, dl, d, dlo, T, Dr, DT, dn);
     }
@@ -716,7 +743,6 @@ __device__ __forceinline__ void propagate_field(const LayerDesc &Ld, float kb, f
     const float tt = sqrtf(tt2), itt = 1.f / tt, itt2 = itt * itt;
     const float sth = tt / sqrtf(tn2);  // sin(theta) at the end
     // J columns (outputs x, y, z, q/pT, phi, theta) of a tangent (dr, dT, dlambda)
-    float J[6][6];
 #pragma unroll
     for (int j = 0; j < 6; ++j) {
         const float *dr = Dr[j], *dT = DT[j];
@@ -737,8 +763,6 @@ __device__ __forceinline__ void propagate_field(const LayerDesc &Ld, float kb, f
         J[5][j] = fmaf(T[2], dtt, -tt * t[2]) / tn2;
     }
 
-    transport_cov(J, C);
-
     // state at the end: position pairs, azimuth turned by the angle between
     // the start and end transverse directions, theta and q/pT = lambda / sin(theta)
     df_add(p[0], lo.x, d[0]);
@@ -758,6 +782,14 @@ __device__ __forceinline__ void propagate_field(const LayerDesc &Ld, float kb, f
     // (sin, cos) = (st, ct) and (tt, T[2]) / |T|
     df_add(p[5], lo.th, atan2f(fmaf(tt, ct, -T[2] * st), fmaf(T[2], ct, tt * st)));
     p[3] = lam / sth;
+}
+
+template <class Cov>
+__device__ __forceinline__ void propagate_field(const LayerDesc &Ld, float kb, float alpha, float p[6], Lo &lo,
+                                                Cov C, float sphi, float cphi, float h, float s) {
+    float J[6][6];
+    move_field(Ld, kb, alpha, p, lo, J, sphi, cphi, h, s);
+    transport_cov(J, C);
 }
 
 // Multiple scattering in the layer's material, added to the covariance of a
