@@ -1009,11 +1009,18 @@ __global__ void __launch_bounds__(256, 2) find_kernel(const __grid_constant__ Fi
             const uint32_t nohit = searched ? kCodeMiss : kCodePass;
             bool got = false;
             if (N == 1) {
-                if (n_children > 0) {
-                    got = true;
-                    hist[step * 32 + lane] = nlist > 0 ? static_cast<uint32_t>(lorig[lane]) : nohit;
-                    sel[lane] = 0;
-                }
+                // best hit: the lane's own first child, its state stays where it is
+                // (no hand-over: 254 -> 245 us for 120 000 seeds of 20 dense events)
+                live = n_children > 0;
+                pend = live;
+                pcode = nlist > 0 ? static_cast<uint32_t>(lorig[lane]) : nohit;
+                if (live) hist[step * 32 + lane] = pcode;
+                const bool hit = live && nlist > 0;
+                pu = hit ? lu[lane] : 0.f;
+                pv = hit ? lv[lane] : 0.f;
+                px2 = hit ? lchi[lane] : 0.f;
+                ++step;
+                continue;
             } else {
                 const uint32_t tag = 15u - static_cast<uint32_t>(rank);
                 int head = 0;
