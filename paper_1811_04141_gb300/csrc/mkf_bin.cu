@@ -51,6 +51,7 @@ __global__ void __launch_bounds__(kBinThreads) bin_keys_kernel(const __grid_cons
     // (binning of the 512 uneven dense events: 2.52 ms before, 2.03 ms after;
     // issuing the thread's histogram adds together then brought it to 1.94 ms)
     __shared__ LayerDesc SL[kMaxLayers];
+    after_previous();
     {
         const int *src = reinterpret_cast<const int *>(A.G.L);
         int *dst = reinterpret_cast<int *>(SL);
@@ -181,6 +182,7 @@ __device__ int block_scan_tile(const int32_t *in, int64_t n, int64_t base, int v
 }
 
 __global__ void __launch_bounds__(kScanThreads) scan_tiles_kernel(const int32_t *counts, int64_t n, int32_t *blocksums) {
+    after_previous();
     int vals[kScanPerThread];
     int t = block_scan_tile(counts, n, (int64_t)blockIdx.x * kScanTile, vals);
     if (threadIdx.x == 0) blocksums[blockIdx.x] = t;
@@ -195,6 +197,7 @@ __global__ void __launch_bounds__(kScanThreads) scan_write_kernel(int32_t *count
                                                                 int64_t nblk, int32_t *offsets, bool zero_counts) {
     __shared__ int red[kScanThreads / 32];
     __shared__ int add_s;
+    after_previous();
     int part = 0;
     for (int64_t b = threadIdx.x; b < (int64_t)blockIdx.x; b += kScanThreads) part += tilesums[b];
 #pragma unroll
@@ -239,6 +242,7 @@ __global__ void __launch_bounds__(kBinThreads) scatter_kernel(const float *X, co
                                                               const int32_t *key, const uint8_t *layer8, int32_t n_hits,
                                                               unsigned long long disk_mask, const int32_t *offsets,
                                                               float4 *rec, int32_t *inv) {
+    after_previous();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n_hits) return;
     const int k = key[i];
@@ -266,6 +270,7 @@ constexpr int kSortBins = 256;
 
 __global__ void __launch_bounds__(kSortBins) bin_sort_kernel(const int32_t *offsets, int64_t n_bins, float4 *rec,
                                                              int32_t *inv) {
+    after_previous();
     const int64_t b = (int64_t)blockIdx.x * kSortBins + threadIdx.x;
     if (b >= n_bins) return;
     const int s = offsets[b], e = offsets[b + 1];
@@ -351,25 +356,23 @@ mkf_status run_binning(mkf_ctx *ctx, const float *xyz, const int32_t *layer, con
         A.counts = counts;
         A.slot = inv;
         A.fault = ctx->fault;
-        bin_keys_kernel<<<(n_hits + kBinThreads * kBinItems - 1) / (kBinThreads * kBinItems), kBinThreads, 0, s>>>(A);
-        MKF_CUDA_TRY(cudaGetLastError());
+        MKF_CUDA_TRY(mkf_launch(bin_keys_kernel, (n_hits + kBinThreads * kBinItems - 1) / (kBinThreads * kBinItems),
+                                kBinThreads, 0, s, A));
     }
     const int64_t nblk = (n_bins + kScanTile - 1) / kScanTile;
-    scan_tiles_kernel<<<(unsigned)nblk, kScanThreads, 0, s>>>(counts, n_bins, tilesums);
-    MKF_CUDA_TRY(cudaGetLastError());
-    scan_write_kernel<<<(unsigned)nblk, kScanThreads, 0, s>>>(counts, n_bins, tilesums, nblk, offsets, true);
-    MKF_CUDA_TRY(cudaGetLastError());
+    MKF_CUDA_TRY(mkf_launch(scan_tiles_kernel, (unsigned)nblk, kScanThreads, 0, s, counts, n_bins, tilesums));
+    MKF_CUDA_TRY(mkf_launch(scan_write_kernel, (unsigned)nblk, kScanThreads, 0, s, counts, n_bins, tilesums, nblk, offsets,
+                            true));
     if (n_hits > 0) {
         unsigned long long disk_mask = 0;
         for (int l = 0; l < ctx->geom.n_layers; ++l)
             if (ctx->geom.L[l].kind == 1) disk_mask |= 1ull << l;
-        scatter_kernel<<<(n_hits + kBinThreads - 1) / kBinThreads, kBinThreads, 0, s>>>(xyz, xyz + n_hits, xyz + 2 * (int64_t)n_hits, key, layer8,
-                                                           n_hits, disk_mask, offsets, rec, inv);
-        MKF_CUDA_TRY(cudaGetLastError());
+        MKF_CUDA_TRY(mkf_launch(scatter_kernel, (n_hits + kBinThreads - 1) / kBinThreads, kBinThreads, 0, s, xyz,
+                                xyz + n_hits, xyz + 2 * (int64_t)n_hits, key, layer8, n_hits, disk_mask, offsets, rec,
+                                inv));
         if (order_bins) {
-            bin_sort_kernel<<<(unsigned)((n_bins + kSortBins - 1) / kSortBins), kSortBins, 0, s>>>(offsets, n_bins, rec,
-                                                                                                   inv);
-            MKF_CUDA_TRY(cudaGetLastError());
+            MKF_CUDA_TRY(mkf_launch(bin_sort_kernel, (unsigned)((n_bins + kSortBins - 1) / kSortBins), kSortBins, 0, s,
+                                    offsets, n_bins, rec, inv));
         }
     }
     return MKF_OK;
@@ -386,12 +389,10 @@ mkf_status mkf_run_scan(cudaStream_t s, const int32_t *counts, int64_t n, int32_
         MKF_CUDA_TRY(cudaMemsetAsync(offsets, 0, sizeof(int32_t), s));
         return MKF_OK;
     }
-    scan_tiles_kernel<<<(unsigned)nblk, kScanThreads, 0, s>>>(counts, n, tilesums);
-    MKF_CUDA_TRY(cudaGetLastError());
+    MKF_CUDA_TRY(mkf_launch(scan_tiles_kernel, (unsigned)nblk, kScanThreads, 0, s, counts, n, tilesums));
     // the counts stay as they are (the caller hands out places from them)
-    scan_write_kernel<<<(unsigned)nblk, kScanThreads, 0, s>>>(const_cast<int32_t *>(counts), n, tilesums, nblk, offsets,
-                                                              false);
-    MKF_CUDA_TRY(cudaGetLastError());
+    MKF_CUDA_TRY(mkf_launch(scan_write_kernel, (unsigned)nblk, kScanThreads, 0, s, const_cast<int32_t *>(counts), n,
+                            tilesums, nblk, offsets, false));
     return MKF_OK;
 }
 

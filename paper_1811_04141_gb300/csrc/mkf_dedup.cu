@@ -25,6 +25,7 @@ constexpr int kThreads = 256;
 // 44 000 tracks of 23 rows).
 __global__ void __launch_bounds__(kThreads) count_kernel(const int32_t *lists, int32_t rows, int32_t n,
                                                          int32_t n_hits, int32_t *cnt) {
+    after_previous();
     const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x;
     if (t >= (int64_t)rows * n) return;
     const int32_t h = lists[t];
@@ -35,6 +36,7 @@ __global__ void __launch_bounds__(kThreads) count_kernel(const int32_t *lists, i
 // counters are ready for the next call.
 __global__ void __launch_bounds__(kThreads) fill_kernel(const int32_t *lists, int32_t rows, int32_t n, int32_t n_hits,
                                                         const int32_t *off, int32_t *cnt, int32_t *items) {
+    after_previous();
     const int64_t t = (int64_t)blockIdx.x * kThreads + threadIdx.x;
     if (t >= (int64_t)rows * n) return;
     const int32_t h = lists[t];
@@ -86,6 +88,7 @@ __global__ void __launch_bounds__(kThreads) seeds_decide_kernel(const int32_t *s
                                                                 const float *par, double max_dqpt, double max_deta,
                                                                 double max_dphi, const int32_t *off,
                                                                 const int32_t *items, int32_t *keep) {
+    after_previous();
     const int32_t i = blockIdx.x * kThreads + threadIdx.x;
     if (i >= n) return;
     // the three hits' ranges at once: most seeds share none and end there
@@ -124,6 +127,7 @@ __global__ void __launch_bounds__(kThreads) tracks_decide_kernel(const int32_t *
                                                                  int32_t n_hits, const int32_t *nh, const float *chi2,
                                                                  float min_frac, const int32_t *off,
                                                                  const int32_t *items, int32_t *keep) {
+    after_previous();
     const int32_t i = blockIdx.x * kThreads + threadIdx.x;
     if (i >= n) return;
     const int32_t ni = nh[i];
@@ -189,14 +193,12 @@ mkf_status build_index(mkf_ctx *ctx, const int32_t *lists, int32_t rows, int32_t
     MKF_CUDA_TRY(cudaMemsetAsync(cnt, 0, sizeof(int32_t) * (size_t)n_hits, s));
     const unsigned blocks = static_cast<unsigned>((pairs + kThreads - 1) / kThreads);
     if (pairs > 0) {
-        count_kernel<<<blocks, kThreads, 0, s>>>(lists, rows, n, n_hits, cnt);
-        MKF_CUDA_TRY(cudaGetLastError());
+        MKF_CUDA_TRY(mkf_launch(count_kernel, blocks, kThreads, 0, s, lists, rows, n, n_hits, cnt));
     }
     const mkf_status ss = mkf_run_scan(s, cnt, n_hits, ts, off);
     if (ss != MKF_OK) return ss;
     if (pairs > 0) {
-        fill_kernel<<<blocks, kThreads, 0, s>>>(lists, rows, n, n_hits, off, cnt, items);
-        MKF_CUDA_TRY(cudaGetLastError());
+        MKF_CUDA_TRY(mkf_launch(fill_kernel, blocks, kThreads, 0, s, lists, rows, n, n_hits, off, cnt, items));
     }
     *off_out = off;
     *items_out = items;
@@ -219,9 +221,8 @@ extern "C" mkf_status mkf_seeds_clean(mkf_ctx *ctx, const int32_t *seed_hits, in
     const int32_t *off = nullptr, *items = nullptr;
     const mkf_status st = build_index(ctx, seed_hits, 3, n_seeds, n_hits, &off, &items);
     if (st != MKF_OK) return st;
-    seeds_decide_kernel<<<(n_seeds + kThreads - 1) / kThreads, kThreads, 0, ctx->stream>>>(
-        seed_hits, n_seeds, n_hits, seed_par, max_dqpt, max_deta, max_dphi, off, items, keep);
-    MKF_CUDA_TRY(cudaGetLastError());
+    MKF_CUDA_TRY(mkf_launch(seeds_decide_kernel, (n_seeds + kThreads - 1) / kThreads, kThreads, 0, ctx->stream, seed_hits,
+                            n_seeds, n_hits, seed_par, max_dqpt, max_deta, max_dphi, off, items, keep));
     return MKF_OK;
 }
 
@@ -240,8 +241,7 @@ extern "C" mkf_status mkf_tracks_dedup(mkf_ctx *ctx, const int32_t *hit_idx, int
     const int32_t *off = nullptr, *items = nullptr;
     const mkf_status st = build_index(ctx, hit_idx, max_hits, n, n_hits, &off, &items);
     if (st != MKF_OK) return st;
-    tracks_decide_kernel<<<(n + kThreads - 1) / kThreads, kThreads, 0, ctx->stream>>>(
-        hit_idx, max_hits, n, n_hits, track_nhits, chi2, min_frac, off, items, keep);
-    MKF_CUDA_TRY(cudaGetLastError());
+    MKF_CUDA_TRY(mkf_launch(tracks_decide_kernel, (n + kThreads - 1) / kThreads, kThreads, 0, ctx->stream, hit_idx, max_hits,
+                            n, n_hits, track_nhits, chi2, min_frac, off, items, keep));
     return MKF_OK;
 }

@@ -485,7 +485,11 @@ template <int kPhys>
 __global__ void __launch_bounds__(128) seed_kernel(const __grid_constant__ FindArgs A) {
     constexpr bool kParamField = kPhys == 2;
     constexpr int kSq = kPhys >= 1 ? 9 : 5;  // square-root columns (two per layer of material)
+    after_previous();
     const int li = blockIdx.x * blockDim.x + threadIdx.x;
+    // the finder's work counter, read after this kernel (with material a memset
+    // comes before it anyway and sets it)
+    if (kPhys == 0 && li == 0) *A.work_counter = 0;
     if (li >= seeds_in_call(A)) return;
     const int t = A.seed_list ? A.seed_list[li] : li;  // the seed
     if (t < 0 || t >= A.n_seeds) {
@@ -731,6 +735,7 @@ __global__ void __launch_bounds__(256, 2) find_kernel(const __grid_constant__ Fi
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ Geom SG;
     __shared__ float WS[MKF_MLP_PARAMS];
+    after_previous();
     {
         const int *src = reinterpret_cast<const int *>(&A.G);
         int *dst = reinterpret_cast<int *>(&SG);
@@ -1117,6 +1122,7 @@ __global__ void __launch_bounds__(256, 2) find_kernel(const __grid_constant__ Fi
 __global__ void __launch_bounds__(256) order_scatter_kernel(const int32_t *key, const int32_t *pos,
                                                             const int32_t *offsets, int n, const int32_t *list,
                                                             const int32_t *list_count, int32_t *order) {
+    after_previous();
     const int li = blockIdx.x * blockDim.x + threadIdx.x;
     const int count = list ? min(max(*list_count, 0), n) : n;
     if (li >= count) return;
@@ -1170,6 +1176,7 @@ __device__ __forceinline__ int block_exclusive_scan(int v, int *warp_sums, int *
 __global__ void __launch_bounds__(kWhereThreads) where_count_kernel(const uint32_t *status, int n, uint32_t bits,
                                                                     int32_t *tile_counts) {
     __shared__ int warp_sums[kWhereThreads / 32];
+    after_previous();
     bool f[kWherePer];
     const int c = where_flags(status, n, bits, blockIdx.x * kWhereTile + threadIdx.x * kWherePer, f);
     int tot;
@@ -1181,6 +1188,7 @@ __global__ void __launch_bounds__(kWhereThreads) where_count_kernel(const uint32
 __global__ void __launch_bounds__(kWhereThreads) where_scan_kernel(int32_t *tile_counts, int n_tiles,
                                                                    int32_t *count) {
     __shared__ int warp_sums[kWhereThreads / 32];
+    after_previous();
     int carry = 0;
     for (int base = 0; base < n_tiles; base += kWhereThreads) {
         const int i = base + threadIdx.x;
@@ -1197,6 +1205,7 @@ __global__ void __launch_bounds__(kWhereThreads) where_scan_kernel(int32_t *tile
 __global__ void __launch_bounds__(kWhereThreads) where_write_kernel(const uint32_t *status, int n, uint32_t bits,
                                                                     const int32_t *tile_offsets, int32_t *list) {
     __shared__ int warp_sums[kWhereThreads / 32];
+    after_previous();
     bool f[kWherePer];
     const int first = blockIdx.x * kWhereTile + threadIdx.x * kWherePer;
     const int c = where_flags(status, n, bits, first, f);
@@ -1590,7 +1599,6 @@ extern "C" mkf_status mkf_find(mkf_ctx *ctx, const mkf_hitbins *bins, const int3
     if (params->mlp_mode != 0 && params->mlp_mode != 1) return MKF_ERR_ARG;
     if (params->mlp_mode == 1 && (!params->mlp_bf16 || params->feat_out)) return MKF_ERR_ARG;
     if (params->seed_order != 0 && params->seed_order != 1) return MKF_ERR_ARG;
-    const bool grouped = params->seed_order == 0;
     A.seed_list = params->seed_list;
     A.seed_count = params->seed_count;
     A.mlp_mode = params->mlp_mode;
@@ -1628,66 +1636,6 @@ extern "C" mkf_status mkf_find(mkf_ctx *ctx, const mkf_hitbins *bins, const int3
                                               static_cast<int>(wide_smem_bytes(MKF_MAX_LAYERS, MKF_MAX_NBEST))));
         ctx->find_smem_attr = want;
     }
-    void *scratch = nullptr;
-    const size_t seed_bytes = ((sizeof(float) * (size_t)kSeedFields * n_seeds + 255) / 256) * 256;
-    // the plain finder's first step runs in the seed kernel (one thread per
-    // seed instead of one busy lane of N); its candidates go through the beam
-    A.step1 = learned ? 0 : 1;
-    const size_t beam_bytes =
-        A.step1 ? ((sizeof(float) * (size_t)kListFields * n_seeds * N + 255) / 256) * 256 : 0;
-    // the processing order (grouped by event and |eta|): keys, places, order, key counts
-    const int n_keys = bins->n_events * kOrderBuckets;
-    const size_t order_bytes =
-        grouped ? ((sizeof(int32_t) * (3 * (size_t)n_seeds + n_keys + 1) + 255) / 256) * 256 : 0;
-    // seeds with a wide window go to find_wide_kernel: with material, in the
-    // plain finder and in the cascade's best-hit pass
-    const bool leave = learned ? phys == 1 && params->mlp_mode == 1 && N == 1 : phys >= 1;
-    const size_t wide_bytes = leave ? ((sizeof(int32_t) * (size_t)n_seeds + 255) / 256) * 256 : 0;
-    mkf_status st = mkf_scratch(ctx, seed_bytes + beam_bytes + order_bytes + wide_bytes + 256, &scratch);
-    if (st != MKF_OK) return st;
-    A.seedbuf = static_cast<float *>(scratch);
-    A.beam = A.step1 ? reinterpret_cast<float *>(static_cast<char *>(scratch) + seed_bytes) : nullptr;
-    char *const tail = static_cast<char *>(scratch) + seed_bytes + beam_bytes + order_bytes;
-    A.work_counter = reinterpret_cast<int32_t *>(tail + wide_bytes);
-    A.wide_list = leave ? reinterpret_cast<int32_t *>(tail) : nullptr;
-    A.wide_count = A.work_counter + 1;
-    A.wide_next = A.work_counter + 2;
-    const int64_t wide_bins = kWideHits * bins->n_bins / std::max(1, bins->n_hits);
-    A.wide_bins = static_cast<int32_t>(std::min<int64_t>(std::max<int64_t>(wide_bins, 1), 1 << 30));
-    int32_t *order = nullptr;
-    A.order_key = A.order_pos = A.order_counts = nullptr;
-    if (grouped) {
-        int32_t *ob = reinterpret_cast<int32_t *>(static_cast<char *>(scratch) + seed_bytes + beam_bytes);
-        A.order_key = ob;
-        A.order_pos = ob + n_seeds;
-        order = ob + 2 * (size_t)n_seeds;
-        A.order_counts = ob + 3 * (size_t)n_seeds;
-        MKF_CUDA_TRY(cudaMemsetAsync(A.order_counts, 0, sizeof(int32_t) * (n_keys + 1), ctx->stream));
-    }
-    A.event_times = reinterpret_cast<unsigned long long *>(params->event_times);
-    // the list of seeds left and the counters behind it
-    MKF_CUDA_TRY(cudaMemsetAsync(tail, 0, wide_bytes + 3 * sizeof(int32_t), ctx->stream));
-    if (A.event_times) {
-        MKF_CUDA_TRY(cudaMemsetAsync(A.event_times, 0, sizeof(uint64_t) * bins->n_events, ctx->stream));
-        MKF_CUDA_TRY(cudaMemsetAsync(A.event_times + bins->n_events, 0xff, sizeof(uint64_t), ctx->stream));
-    }
-    switch (phys) {
-        case 0: seed_kernel<0><<<(n_seeds + 127) / 128, 128, 0, ctx->stream>>>(A); break;
-        case 1: seed_kernel<1><<<(n_seeds + 127) / 128, 128, 0, ctx->stream>>>(A); break;
-        default: seed_kernel<2><<<(n_seeds + 127) / 128, 128, 0, ctx->stream>>>(A); break;
-    }
-    MKF_CUDA_TRY(cudaGetLastError());
-    if (grouped) {
-        // key counts -> offsets (the total, n_seeds, lands in the last entry),
-        // then the order; the finder takes the seeds through it
-        where_scan_kernel<<<1, kWhereThreads, 0, ctx->stream>>>(A.order_counts, n_keys, A.order_counts + n_keys);
-        order_scatter_kernel<<<(n_seeds + 255) / 256, 256, 0, ctx->stream>>>(
-            A.order_key, A.order_pos, A.order_counts, n_seeds, A.seed_list, A.seed_count, order);
-        MKF_CUDA_TRY(cudaGetLastError());
-        A.order_key = nullptr;  // the finder writes no keys
-        A.seed_list = order;
-        A.seed_count = A.order_counts + n_keys;
-    }
     // persistent grid: as many blocks as fit on the device at once, or fewer
     const int spw = 32 / N;
     const int seeds_per_block = spw * (threads / 32);
@@ -1703,24 +1651,71 @@ extern "C" mkf_status mkf_find(mkf_ctx *ctx, const mkf_hitbins *bins, const int3
     }
     const int per_sm = ctx->find_occ_blocks[vi];
     const int blocks = std::max(1, std::min(need, std::max(1, per_sm) * ctx->num_sms));
-    void *kargs[1] = {&A};
-    MKF_CUDA_TRY(cudaLaunchKernel(kfn, dim3(blocks), dim3(threads), kargs, smem, ctx->stream));
-    if (leave) {
-        // how many seeds were left is known on the device only: the blocks that
-        // find none exit at once
-        const int wide_blocks = std::min(n_seeds, 3 * ctx->num_sms);
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(wide_blocks);
-        cfg.blockDim = dim3(wide_threads(N));
-        cfg.dynamicSmemBytes = wide_smem_bytes(ctx->geom.n_layers, N);
-        cfg.stream = ctx->stream;
-        cudaLaunchAttribute attr = {};
-        attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr.val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = &attr;
-        cfg.numAttrs = 1;
-        MKF_CUDA_TRY(cudaLaunchKernelExC(&cfg, wfn, kargs));
+    // seeds that all have a warp at once are taken in the input order: nothing
+    // waits behind a long one there, and the two kernels that make the order
+    // would only come on top (2000 seeds: 79 us with them, 67 without; at the
+    // line, 7000 to 9000 seeds at N = 10, either way gains what it should)
+    const bool grouped = params->seed_order == 0 && need > blocks;
+    void *scratch = nullptr;
+    const size_t seed_bytes = ((sizeof(float) * (size_t)kSeedFields * n_seeds + 255) / 256) * 256;
+    // the plain finder's first step runs in the seed kernel (one thread per
+    // seed instead of one busy lane of N); its candidates go through the beam
+    A.step1 = learned ? 0 : 1;
+    const size_t beam_bytes =
+        A.step1 ? ((sizeof(float) * (size_t)kListFields * n_seeds * N + 255) / 256) * 256 : 0;
+    // the processing order (grouped by event and |eta|): keys, places, order
+    const int n_keys = bins->n_events * kOrderBuckets;
+    const size_t order_bytes = grouped ? ((sizeof(int32_t) * 3 * (size_t)n_seeds + 255) / 256) * 256 : 0;
+    // seeds with a wide window go to find_wide_kernel: with material, in the
+    // plain finder and in the cascade's best-hit pass
+    const bool leave = learned ? phys == 1 && params->mlp_mode == 1 && N == 1 : phys >= 1;
+    // words that start at zero: the list of those seeds and its counters, the
+    // order's key counts (and their total)
+    const size_t zero_words = leave ? (size_t)n_seeds + 2 : 0;
+    const size_t tail_bytes = sizeof(int32_t) * (zero_words + (grouped ? n_keys + 1 : 0) + 1);
+    mkf_status st = mkf_scratch(ctx, seed_bytes + beam_bytes + order_bytes + tail_bytes + 256, &scratch);
+    if (st != MKF_OK) return st;
+    A.seedbuf = static_cast<float *>(scratch);
+    A.beam = A.step1 ? reinterpret_cast<float *>(static_cast<char *>(scratch) + seed_bytes) : nullptr;
+    int32_t *const ob = reinterpret_cast<int32_t *>(static_cast<char *>(scratch) + seed_bytes + beam_bytes);
+    int32_t *const tail = reinterpret_cast<int32_t *>(static_cast<char *>(scratch) + seed_bytes + beam_bytes + order_bytes);
+    A.wide_list = leave ? tail : nullptr;
+    A.wide_count = leave ? tail + n_seeds : nullptr;
+    A.wide_next = leave ? tail + n_seeds + 1 : nullptr;
+    const int64_t wide_bins = kWideHits * bins->n_bins / std::max(1, bins->n_hits);
+    A.wide_bins = static_cast<int32_t>(std::min<int64_t>(std::max<int64_t>(wide_bins, 1), 1 << 30));
+    A.order_key = grouped ? ob : nullptr;
+    A.order_pos = grouped ? ob + n_seeds : nullptr;
+    int32_t *const order = grouped ? ob + 2 * (size_t)n_seeds : nullptr;
+    A.order_counts = grouped ? tail + zero_words : nullptr;
+    A.work_counter = tail + zero_words + (grouped ? n_keys + 1 : 0);
+    if (phys > 0 || grouped)  // (else the seed kernel clears the work counter, the only one)
+        MKF_CUDA_TRY(cudaMemsetAsync(tail, 0, tail_bytes, ctx->stream));
+    A.event_times = reinterpret_cast<unsigned long long *>(params->event_times);
+    if (A.event_times) {
+        MKF_CUDA_TRY(cudaMemsetAsync(A.event_times, 0, sizeof(uint64_t) * bins->n_events, ctx->stream));
+        MKF_CUDA_TRY(cudaMemsetAsync(A.event_times + bins->n_events, 0xff, sizeof(uint64_t), ctx->stream));
     }
+    MKF_CUDA_TRY(mkf_launch(phys == 0 ? seed_kernel<0> : phys == 1 ? seed_kernel<1> : seed_kernel<2>,
+                            (n_seeds + 127) / 128, 128, 0, ctx->stream, A));
+    if (grouped) {
+        // key counts -> offsets (the total, n_seeds, lands in the last entry),
+        // then the order; the finder takes the seeds through it
+        MKF_CUDA_TRY(mkf_launch(where_scan_kernel, 1, kWhereThreads, 0, ctx->stream, A.order_counts, n_keys,
+                                A.order_counts + n_keys));
+        MKF_CUDA_TRY(mkf_launch(order_scatter_kernel, (n_seeds + 255) / 256, 256, 0, ctx->stream, A.order_key, A.order_pos,
+                                A.order_counts, n_seeds, A.seed_list, A.seed_count, order));
+        A.order_key = nullptr;  // the finder writes no keys
+        A.seed_list = order;
+        A.seed_count = A.order_counts + n_keys;
+    }
+    typedef void (*FindFn)(FindArgs);
+    MKF_CUDA_TRY(mkf_launch((FindFn)kfn, blocks, threads, smem, ctx->stream, A));
+    if (leave)
+        // how many seeds were left is known on the device only: the blocks that
+        // find none end at once
+        MKF_CUDA_TRY(mkf_launch((FindFn)wfn, std::min(n_seeds, 3 * ctx->num_sms), wide_threads(N),
+                                wide_smem_bytes(ctx->geom.n_layers, N), ctx->stream, A));
     return MKF_OK;
 }
 
@@ -1740,9 +1735,8 @@ extern "C" mkf_status mkf_seeds_where(mkf_ctx *ctx, const uint32_t *status, int3
     mkf_status st = mkf_scratch(ctx, sizeof(int32_t) * (size_t)n_tiles, &scratch);
     if (st != MKF_OK) return st;
     int32_t *tiles = static_cast<int32_t *>(scratch);
-    where_count_kernel<<<n_tiles, kWhereThreads, 0, ctx->stream>>>(status, n, bits, tiles);
-    where_scan_kernel<<<1, kWhereThreads, 0, ctx->stream>>>(tiles, n_tiles, seed_count);
-    where_write_kernel<<<n_tiles, kWhereThreads, 0, ctx->stream>>>(status, n, bits, tiles, seed_list);
-    MKF_CUDA_TRY(cudaGetLastError());
+    MKF_CUDA_TRY(mkf_launch(where_count_kernel, n_tiles, kWhereThreads, 0, ctx->stream, status, n, bits, tiles));
+    MKF_CUDA_TRY(mkf_launch(where_scan_kernel, 1, kWhereThreads, 0, ctx->stream, tiles, n_tiles, seed_count));
+    MKF_CUDA_TRY(mkf_launch(where_write_kernel, n_tiles, kWhereThreads, 0, ctx->stream, status, n, bits, tiles, seed_list));
     return MKF_OK;
 }
