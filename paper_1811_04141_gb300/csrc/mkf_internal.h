@@ -79,10 +79,10 @@ struct mkf_hitbins {
 // that small), the chain of twenty kernels around finding on 20 such events 517
 // -> 479 us.
 template <typename... P, typename... A>
-inline cudaError_t mkf_launch(void (*kernel)(P...), unsigned blocks, unsigned threads, size_t smem, cudaStream_t s,
+inline cudaError_t mkf_launch(void (*kernel)(P...), dim3 blocks, unsigned threads, size_t smem, cudaStream_t s,
                               A... args) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(blocks);
+    cfg.gridDim = blocks;
     cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;

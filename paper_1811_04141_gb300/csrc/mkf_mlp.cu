@@ -70,7 +70,8 @@ __global__ void __launch_bounds__(128) forward_kernel(const uint16_t *wb, const 
 // work on a chunk, and nothing per sample goes through global memory: the
 // activations and gradients written there by one kernel and read back by the
 // next, one load per addition, made a training step of 4096 samples take 108 us
-// (four kernels; 16.3 us with this one and finish_kernel, bit for bit the same).
+// (four kernels; 16.3 us with this one and finish_kernel, 12.1 us when both are
+// launched while the kernel before them runs; bit for bit the same).
 constexpr int kSlice = 8;
 constexpr int kSlices = kHid / kSlice;
 constexpr int kRow = kChunk + 4;  // a row of the transposed tiles: 16-byte aligned, rows 4 banks apart
@@ -96,6 +97,7 @@ __global__ void __launch_bounds__(kChunk) chunk_grad_kernel(const uint16_t *wb, 
     __shared__ __align__(16) float gs[kChunk];
     __shared__ __align__(16) float ls[kChunk];
     __shared__ __align__(16) float ws[kP + 3];
+    after_previous();
     const int tid = threadIdx.x;
     const int j0 = blockIdx.x * kSlice;
     const int s0 = blockIdx.y * kChunk, ns = min(kChunk, n - s0);
@@ -173,11 +175,15 @@ __global__ void __launch_bounds__(kChunk) chunk_grad_kernel(const uint16_t *wb, 
     part[(int64_t)blockIdx.y * (kP + 1) + p] = acc.sum;
 }
 
-// Sum the chunk partials in chunk order; optionally apply Adam.
+// Sum the chunk partials in chunk order; optionally apply Adam.  Bound: latency;
+// what needs no partial (the bias corrections' powers) is done before the wait.
 __global__ void __launch_bounds__(128) finish_kernel(const float *part, int nchunks, int n, float *grad, float *loss,
                                                      float *w, float *m, float *v, int t, mkf_adam hp, uint16_t *wb) {
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p > kP) return;
+    const float bias1 = 1.f - powf(hp.beta1, static_cast<float>(t));
+    const float bias2 = 1.f - powf(hp.beta2, static_cast<float>(t));
+    after_previous();
     KahanSum acc;
 #pragma unroll 8
     for (int c = 0; c < nchunks; ++c) acc.add(part[(int64_t)c * (kP + 1) + p]);
@@ -192,8 +198,8 @@ __global__ void __launch_bounds__(128) finish_kernel(const float *part, int nchu
         const float vv = hp.beta2 * v[p] + (1.f - hp.beta2) * sum * sum;
         m[p] = mm;
         v[p] = vv;
-        const float mh = mm / (1.f - powf(hp.beta1, static_cast<float>(t)));
-        const float vh = vv / (1.f - powf(hp.beta2, static_cast<float>(t)));
+        const float mh = mm / bias1;
+        const float vh = vv / bias2;
         const float nw = w[p] - hp.lr * mh / (sqrtf(vh) + hp.eps);
         w[p] = nw;
         wb[p] = to_bf16(nw);
@@ -209,11 +215,11 @@ mkf_status run_grad(mkf_ctx *ctx, const uint16_t *wb, const float *feat, const f
     if (st != MKF_OK) return st;
     float *part = static_cast<float *>(scratch);
     cudaStream_t s = ctx->stream;
-    chunk_grad_kernel<<<dim3(kSlices, nchunks), kChunk, 0, s>>>(wb, wb ? nullptr : w, feat, label, n, part);
-    MKF_CUDA_TRY(cudaGetLastError());
+    MKF_CUDA_TRY(mkf_launch(chunk_grad_kernel, dim3(kSlices, nchunks), kChunk, 0, s, wb, wb ? nullptr : w, feat, label,
+                            n, part));
     mkf_adam h = hp ? *hp : mkf_adam{0.f, 0.f, 0.f, 0.f};
-    finish_kernel<<<(kP + 1 + 127) / 128, 128, 0, s>>>(part, nchunks, n, grad, loss, w, m, v, t, h, wb_out);
-    MKF_CUDA_TRY(cudaGetLastError());
+    MKF_CUDA_TRY(mkf_launch(finish_kernel, (kP + 1 + 127) / 128, 128, 0, s, part, nchunks, n, grad, loss, w, m, v, t, h,
+                            wb_out));
     return MKF_OK;
 }
 
