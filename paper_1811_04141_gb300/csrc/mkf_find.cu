@@ -324,11 +324,20 @@ struct Expansion {
 // material, N = 10: 3.7 ms with and 1.1 ms without the 3000 widest of 48 000
 // seeds), so the variants with material leave a seed to find_wide_kernel, which
 // gives every candidate several lanes, as soon as one of its windows holds about
-// this many hits (A.wide_bins bins at the call's mean occupancy).  Measured on
-// that call and on a learned cascade over 16 such events: 77 hits 2.2 / 3.3 ms,
-// 128 1.9 / 2.6, 205 1.8 / 2.3, 320 1.8 / 2.3; by phi bins alone (16 to 48)
-// 1.8-2.1 / 2.4-2.9.
-constexpr int kWideHits = 256;
+// wide_hits hits (A.wide_bins bins at the call's mean occupancy).  By phi bins
+// alone (16 to 48) the same call takes 1.8-2.1 ms.
+// A seed left costs more work in all than one kept, and gains only at the call's
+// end, so the line rises with the seeds to work on.  Times in ms at 128, 256, 512
+// and 1024 hits, N = 10, against no seed left: 2 dense events (12 000 seeds) 0.72,
+// 0.80, 0.91, 0.95 (0.96); 8 events 1.90, 1.75, 1.79, 1.96 (2.96); 32 events 6.8,
+// 5.8, 5.6, 5.6 (6.8); 128 events 26.2, 22.2, 20.5, 20.5 (21.2).  At N = 1 a lane
+// holds a seed and a warp 32 of them: 256 to 512 at every size (96 000 seeds 1.12,
+// 0.91, 0.91, 0.99; 2.0).  A call on a list of seeds knows its length on the device
+// only and is taken to work on half (a cascade's second pass over 16 such events:
+// 250 hits 2.2 ms, 500 2.4; over 96: 8.4 and 7.9).
+inline int wide_hits(int n_seeds, int n_best, bool listed) {
+    return std::min(std::max(n_seeds / (listed ? 384 : 192), n_best == 1 ? 256 : 128), 512);
+}
 
 // One candidate to its next layer: next-layer choice, propagation and
 // covariance transport, S^-1 and H C, the bins of the chi2 window, and the
@@ -1257,7 +1266,7 @@ __device__ __forceinline__ int next_wide(const FindArgs &A) {
 }
 
 // The finder for the seeds that find_kernel left because of a wide window (see
-// kWideHits): one block per seed, wide_lanes(N) lanes per candidate.  The lanes
+// wide_hits): one block per seed, wide_lanes(N) lanes per candidate.  The lanes
 // of a candidate all hold its state and move it together (the same arithmetic
 // as in find_kernel, so the same bits); they share the phi bins of its window,
 // each with a list of its own, and the lists are merged by N rounds of a minimum
@@ -1682,7 +1691,8 @@ extern "C" mkf_status mkf_find(mkf_ctx *ctx, const mkf_hitbins *bins, const int3
     A.wide_list = leave ? tail : nullptr;
     A.wide_count = leave ? tail + n_seeds : nullptr;
     A.wide_next = leave ? tail + n_seeds + 1 : nullptr;
-    const int64_t wide_bins = kWideHits * bins->n_bins / std::max(1, bins->n_hits);
+    const int64_t wide_bins =
+        wide_hits(n_seeds, N, params->seed_list != nullptr) * bins->n_bins / std::max(1, bins->n_hits);
     A.wide_bins = static_cast<int32_t>(std::min<int64_t>(std::max<int64_t>(wide_bins, 1), 1 << 30));
     A.order_key = grouped ? ob : nullptr;
     A.order_pos = grouped ? ob + n_seeds : nullptr;

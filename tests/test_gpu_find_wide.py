@@ -93,3 +93,24 @@ def test_wide_windows_with_the_gate_and_in_a_graph():
         g["status"] &= ~64
         _same(g, p)
     ctx.close()
+
+
+@pytest.mark.parametrize("times,n_best,listed", [(1, 2, False), (14, 2, False), (40, 2, False), (1, 1, True), (30, 3, True)])
+def test_the_line_over_the_number_of_seeds(times, n_best, listed):
+    """The window size from which seeds are left grows with the call's seeds; the outputs do not change."""
+    b = _batch()
+    ctx = _ctx(b)
+    d = upload(b)
+    mlp = torch.zeros(897, dtype=torch.int16, device="cuda")
+    bins = ctx.hits_bin(d["xyz"], d["layer"], d["event_offsets"])
+    ref = ctx.find(bins, d["seed_hits"], d["seed_event"], n_best=n_best, mlp_bf16=mlp, mlp_tau=-1.0)
+    n0 = d["seed_event"].shape[0]
+    at = torch.arange(n0 * times, device="cuda") % n0
+    kw = {}
+    if listed:
+        kw = dict(seed_list=torch.arange(n0 * times, dtype=torch.int32, device="cuda"),
+                  seed_count=torch.tensor([n0 * times], dtype=torch.int32, device="cuda"))
+    out = ctx.find(bins, d["seed_hits"][:, at].contiguous(), d["seed_event"][at].contiguous(), n_best=n_best, **kw)
+    ctx.sync()
+    _same(out, {k: v[..., at] for k, v in ref.items()})
+    ctx.close()
