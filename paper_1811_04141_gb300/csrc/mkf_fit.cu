@@ -210,7 +210,7 @@ __device__ __forceinline__ bool first_three(const FitArgs &A, int t, int first[3
 // uniform field without material; 1 material effects compiled in (selected
 // when any layer has material); 2 the parameterised field (Runge-Kutta
 // propagation) with the material effects.
-// Bound: issue and instruction fetch (the uniform-field fit: 66 % of issue slots,
+// Bound: issue and instruction fetch (the uniform-field fit: 72 % of issue slots,
 // the hit code is there twice).  Blocks per SM, measured with the row feed:
 // uniform field 6 / 5 / 4: 334 / 322 / 333 us for 10^6 tracks of 10 hits (at 5
 // nothing spills; 336 us before the feed, at 6); material, out and back, 6 / 5 /
