@@ -398,7 +398,8 @@ typedef struct {
      * seed's outputs are left as they are.  The count is read on the device,
      * so a subset chosen by an earlier call (mkf_seeds_where) needs no host
      * round trip; *seed_count above n_seeds is taken as n_seeds, an index out
-     * of range is a device fault (MKF_ERR_DEVICE_CHECK at mkf_sync). */
+     * of range is a device fault (MKF_ERR_DEVICE_CHECK at mkf_sync), an index
+     * listed more than once is found as often, with the same outputs. */
     const int32_t *seed_list;
     const int32_t *seed_count;
     /* With mlp_bf16: 0 prunes as described above; 1 (gate) drops nothing and

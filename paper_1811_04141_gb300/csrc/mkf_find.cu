@@ -72,8 +72,9 @@ struct FindArgs {
     const int32_t *seed_count;
     int32_t mlp_mode;                     // 0 prune, 1 gate (flag MKF_ST_AMBIG, drop nothing)
     // processing order grouped by event and |eta| of the seed (or nullptr):
-    // the seed kernel writes each seed's key and place, order_scatter_kernel
-    // the order the finder's warps take the seeds in
+    // the seed kernel writes the key and place of each seed of the call (by its
+    // index in the call), order_scatter_kernel the order the finder's warps take
+    // the seeds in
     int32_t *order_key, *order_pos, *order_counts;
     // seeds left to find_wide_kernel (or nullptr: none are): entries seed + 1,
     // zero until written; how many were added and how many taken
@@ -575,8 +576,9 @@ __global__ void __launch_bounds__(128) seed_kernel(const __grid_constant__ FindA
     if (A.order_key) {
         const int key = (ev >= 0 && ev < A.n_events ? ev : 0) * kOrderBuckets +
                         (ok ? min(static_cast<int>(fabsf(eta) * 4.f), kOrderBuckets - 1) : 0);
-        A.order_key[t] = key;
-        A.order_pos[t] = atomicAdd(&A.order_counts[key], 1);
+        // by place in the list, not by seed: a seed listed twice has two places
+        A.order_key[li] = key;
+        A.order_pos[li] = atomicAdd(&A.order_counts[key], 1);
     }
     unsigned long long mask = 0;
     int dir = 1;
@@ -1136,7 +1138,8 @@ __global__ void __launch_bounds__(256) order_scatter_kernel(const int32_t *key, 
     const int count = list ? min(max(*list_count, 0), n) : n;
     if (li >= count) return;
     const int t = list ? list[li] : li;
-    if (t >= 0 && t < n) order[offsets[key[t]] + pos[t]] = t;
+    // an entry out of range has no key; every counted entry has a place of its own
+    if (t >= 0 && t < n) order[offsets[key[li]] + pos[li]] = t;
 }
 
 // Ordered compaction of the seeds whose status has any of `bits` (ascending
