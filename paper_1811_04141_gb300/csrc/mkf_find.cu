@@ -1231,6 +1231,10 @@ __global__ void __launch_bounds__(kWhereThreads) where_write_kernel(const uint32
 // steps: at most one per layer + one final step with no layer left
 int find_max_steps(int n_layers) { return n_layers + 2; }
 
+// Dynamic shared memory of a block of the finder: the most a call may ask for
+// (of the 227 KB; the rest covers the geometry and the weights).
+constexpr size_t kFindMaxSmem = 200 * 1024;
+
 size_t find_smem_bytes(int n_layers, int n_best, int threads) {
     const int nwarps = threads / 32;
     return static_cast<size_t>(nwarps) * (find_max_steps(n_layers) * 32 * 4 + n_best * 32 * 16 + 32 * 4);
@@ -1615,9 +1619,7 @@ extern "C" mkf_status mkf_find(mkf_ctx *ctx, const mkf_hitbins *bins, const int3
     A.seed_count = params->seed_count;
     A.mlp_mode = params->mlp_mode;
     const size_t smem = find_smem_bytes(ctx->geom.n_layers, N, threads);
-    if (smem > 200 * 1024) return MKF_ERR_CAPACITY;
-    // raise the kernel's dynamic shared-memory limit only when needed (not during
-    // a stream capture after the first call)
+    if (smem > kFindMaxSmem) return MKF_ERR_CAPACITY;
     const bool learned = params->mlp_bf16 || params->feat_out;
     // material anywhere in the geometry selects the variant with the material
     // effects compiled in, the parameterised field the one with Runge-Kutta
@@ -1639,14 +1641,18 @@ extern "C" mkf_status mkf_find(mkf_ctx *ctx, const mkf_hitbins *bins, const int3
                                  reinterpret_cast<const void *>(find_wide_kernel<false, 2>),
                                  reinterpret_cast<const void *>(find_wide_kernel<true, 1>)};
     const void *wfn = wfns[learned ? 2 : (phys == 2 ? 1 : 0)];
-    if (static_cast<int>(smem) > ctx->find_smem_attr) {
-        const int want = static_cast<int>(std::max<size_t>(smem, 48 * 1024));
+    // the kernels' dynamic shared-memory limit, once per context (not during a
+    // stream capture after the first call).  It belongs to the kernel on the whole
+    // device, so every context sets the same value: one that set what its own call
+    // needs would lower the limit under another context's later calls.
+    if (!ctx->find_smem_set) {
         for (int v = 0; v < 18; ++v)
-            MKF_CUDA_TRY(cudaFuncSetAttribute(kfns[v], cudaFuncAttributeMaxDynamicSharedMemorySize, want));
+            MKF_CUDA_TRY(cudaFuncSetAttribute(kfns[v], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                              static_cast<int>(kFindMaxSmem)));
         for (const void *w : wfns)
             MKF_CUDA_TRY(cudaFuncSetAttribute(w, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               static_cast<int>(wide_smem_bytes(MKF_MAX_LAYERS, MKF_MAX_NBEST))));
-        ctx->find_smem_attr = want;
+        ctx->find_smem_set = 1;
     }
     // persistent grid: as many blocks as fit on the device at once, or fewer
     const int spw = 32 / N;

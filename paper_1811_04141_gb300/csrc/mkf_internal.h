@@ -36,7 +36,7 @@ struct mkf_ctx {
     void *scratch;
     size_t scratch_bytes;
     int num_sms;
-    int find_smem_attr;  // dynamic shared memory the find kernel is configured for
+    int find_smem_set;  // the find kernels' dynamic shared-memory limits are set
     // cached occupancy per finder variant: (plain, learned) x (uniform field,
     // material, parameterised field) x (beam width at run time, 1, 10)
     int find_occ_threads[18], find_occ_smem[18], find_occ_blocks[18];
