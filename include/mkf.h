@@ -479,7 +479,7 @@ mkf_status mkf_mlp_forward(mkf_ctx *ctx, const uint16_t *w_bf16, const float *fe
  * gradient with respect to the (bfloat16-rounded) weights.  feat [n][12],
  * label [n], grad [MKF_MLP_PARAMS], loss [1]: device.  The batch sum runs in a
  * fixed order: the result does not depend on scheduling.
- * Errors: MKF_ERR_ARG, MKF_ERR_CUDA. */
+ * Errors: MKF_ERR_ARG, MKF_ERR_CUDA (also for n > 65535 * 256). */
 mkf_status mkf_mlp_grad(mkf_ctx *ctx, const uint16_t *w_bf16, const float *feat, const float *label, int32_t n,
                         float *grad, float *loss);
 

@@ -65,10 +65,16 @@ struct mkf_hitbins {
     int ordered;        // hits within each bin in ascending original index
 };
 
+// A refused runtime call is an error of the entry point it was made for and of
+// no later one: the runtime's record of it is cleared, or the next call that
+// checks its launches with cudaGetLastError() would report it as its own.
 #define MKF_CUDA_TRY(expr)                                  \
     do {                                                    \
         cudaError_t e_ = (expr);                            \
-        if (e_ != cudaSuccess) return MKF_ERR_CUDA;         \
+        if (e_ != cudaSuccess) {                            \
+            (void)cudaGetLastError();                       \
+            return MKF_ERR_CUDA;                            \
+        }                                                   \
     } while (0)
 
 #ifdef __CUDACC__
