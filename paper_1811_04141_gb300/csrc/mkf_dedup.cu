@@ -120,9 +120,15 @@ __global__ void __launch_bounds__(kThreads) seeds_decide_kernel(const int32_t *s
 // Tracks: drop i when a better track u (more hits, then lower chi2, then lower
 // index) shares at least max(1, min_frac x the shorter one's hit count) hits.
 // Bound: latency of the chain hit -> range -> items -> the other track, taken for
-// several rows together.  The shared hits are counted through the index (a few
-// items per hit) rather than along the other track's list: 92 -> 30 us for
-// 44 000 tracks of 23 rows, a tenth of them duplicates.
+// several rows together.  Whether the other track lists a hit is looked up among
+// the hit's items where these are no more than a list has rows (a few, mostly:
+// 92 -> 30 us for 44 000 tracks of 23 rows, a tenth of them duplicates), else
+// along the other track's list, or the work would grow with the square of the
+// tracks on a hit.  20 000 tracks of 23 rows in groups that share 40 % of their
+// hits, 128 / 1000 tracks a group: 27.5 / 248 ms; 55.4 / 2960 ms by the items
+// alone, 52.6 / 415 ms along the lists alone.  Groups of equal tracks are bound by
+// the best one's walk over every item, one item ahead of its test: 3.8 ms for
+// 1000 a group (4.2 without, 3.95 along the lists alone).
 __global__ void __launch_bounds__(kThreads) tracks_decide_kernel(const int32_t *hit_idx, int32_t rows, int32_t n,
                                                                  int32_t n_hits, const int32_t *nh, const float *chi2,
                                                                  float min_frac, const int32_t *off,
@@ -147,22 +153,31 @@ __global__ void __launch_bounds__(kThreads) tracks_decide_kernel(const int32_t *
 #pragma unroll
         for (int32_t j = 0; j < kBatch; ++j) {
             if (e[j] - b[j] < 2) continue;  // listed by this track only
+            int32_t next = items[b[j]];  // loaded while the one before it is tested
             for (int32_t p = b[j]; p < e[j] && k_; ++p) {
-                const int32_t u = items[p];
+                const int32_t u = next;
+                if (p + 1 < e[j]) next = items[p + 1];
                 if (u == i) continue;
                 const int32_t nu = nh[u];
                 const float cu = chi2[u];
                 const bool better = nu > ni || (nu == ni && (cu < ci || (cu == ci && u < i)));
                 if (!better) continue;
-                // hits of i (as a set) whose items include u; enough of them end
-                // the count
+                // hits of i (as a set) that u lists; enough of them end the
+                // count.  Looked up among the hit's items or, where these are
+                // more than a list has rows, along u's own list.
                 const double need = fmax(1.0, static_cast<double>(min_frac) * min(ni, nu));
                 int32_t shared = 0;
                 for (int32_t a = 0; a < rows && shared < need; ++a) {
                     const int32_t ha = hit_idx[(int64_t)a * n + i];
                     if (ha < 0 || ha >= n_hits) continue;
+                    const int32_t q0 = off[ha], q1 = off[ha + 1];
+                    // one loop for both (a loop each: 7 % slower where few share a hit)
+                    const bool crowded = q1 - q0 > rows;
+                    const int32_t *L = crowded ? hit_idx + u : &items[q0];
+                    const int64_t stride = crowded ? n : 1;
+                    const int32_t len = crowded ? rows : q1 - q0, want = crowded ? ha : u;
                     bool has = false;
-                    for (int32_t q = off[ha]; q < off[ha + 1] && !has; ++q) has = items[q] == u;
+                    for (int32_t c = 0; c < len && !has; ++c, L += stride) has = *L == want;
                     if (has && !listed_before(hit_idx, a, n, i, ha)) ++shared;
                 }
                 if (shared >= need) k_ = false;
