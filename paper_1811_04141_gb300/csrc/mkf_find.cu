@@ -79,7 +79,7 @@ struct FindArgs {
     // seeds left to find_wide_kernel (or nullptr: none are): entries seed + 1,
     // zero until written; how many were added and how many taken
     int32_t *wide_list, *wide_count, *wide_next;
-    int32_t wide_bins;  // bins of a wide window
+    float wide_bins;  // extent of a wide window, in bins
 };
 
 // Seeds are taken by the finder grouped by event and by the |eta| of their
@@ -325,8 +325,7 @@ struct Expansion {
 // material, N = 10: 3.7 ms with and 1.1 ms without the 3000 widest of 48 000
 // seeds), so the variants with material leave a seed to find_wide_kernel, which
 // gives every candidate several lanes, as soon as one of its windows holds about
-// wide_hits hits (A.wide_bins bins at the call's mean occupancy).  By phi bins
-// alone (16 to 48) the same call takes 1.8-2.1 ms.
+// wide_hits hits: its extent in bins (A.wide_bins) at the call's mean occupancy.
 // A seed left costs more work in all than one kept, and gains only at the call's
 // end, so the line rises with the seeds to work on.  Times in ms at 128, 256, 512
 // and 1024 hits, N = 10, against no seed left: 2 dense events (12 000 seeds) 0.72,
@@ -336,9 +335,32 @@ struct Expansion {
 // 0.91, 0.91, 0.99; 2.0).  A call on a list of seeds knows its length on the device
 // only and is taken to work on half (a cascade's second pass over 16 such events:
 // 250 hits 2.2 ms, 500 2.4; over 96: 8.4 and 7.9).
-inline int wide_hits(int n_seeds, int n_best, bool listed) {
-    return std::min(std::max(n_seeds / (listed ? 384 : 192), n_best == 1 ? 256 : 128), 512);
+// 128 hits only where a layer holds 4000 (crowded): in one of 1000 they are as
+// wide as it gets, and the seed is begun anew for nothing (4 events of 2000 tracks
+// and 20 000 noise hits 0.84 ms at 128, 0.73 at 256; 0.80 with none left).  Four
+// times as many in the parameterised field, where a seed begun anew repeats its
+// Runge-Kutta steps (8 events with windows of most of a layer 2.40 ms, 1.87 at
+// four times, 1.85 with none left; dense events the same either way).
+inline int wide_hits(int phys, int n_seeds, int n_best, bool listed, bool crowded) {
+    const int hits = std::min(std::max(n_seeds / (listed ? 384 : 192), n_best > 1 && crowded ? 128 : 256), 512);
+    return phys == 2 ? 4 * hits : hits;
 }
+
+// The same in bins of the call's grid (each layer has its own: n_bins in all).
+inline float wide_bins(int phys, int n_seeds, int n_best, bool listed, int n_hits, int64_t n_bins, int n_events,
+                       int n_layers) {
+    const bool crowded = n_hits / n_layers / std::max(1, n_events) >= 4000;
+    return static_cast<float>(wide_hits(phys, n_seeds, n_best, listed, crowded)) * static_cast<float>(n_bins) /
+           static_cast<float>(std::max(1, n_hits));
+}
+
+// A window is measured by its own extent and not by the bins it touches: on a
+// coarse grid every window touches bins that hold hundreds of hits (8 dense events,
+// N = 10, 16 x 4 bins a layer: 27.8 ms by the bins touched, 5.2 by the extent, 5.7
+// with none left; 1 x 1, 16 small events: 26, 3.25, 3.25; 64 x 8, 4 endcap events
+// 0.27, 0.21, 0.25; 256 x 32 the same).  It is left only if it has phi bins for the
+// lanes that would share it.
+constexpr int kWideMinPhi = 4;
 
 // One candidate to its next layer: next-layer choice, propagation and
 // covariance transport, S^-1 and H C, the bins of the chi2 window, and the
@@ -415,9 +437,13 @@ __device__ __forceinline__ void expand(const FindArgs &A, const Geom &G, int ev,
     const float zhi_f = fminf(fmaxf(floorf((zc + wz - Ld.lo) * Ld.zr_scale), 0.f), Ld.nzr - 1.f);
     const int zb_lo = static_cast<int>(zlo_f), zb_hi = static_cast<int>(zhi_f);
     const int ebase = ev * G.bins_per_event + Ld.bin_base;
-    if (kLeave && A.wide_list && nphib * (zb_hi - zb_lo + 1) >= A.wide_bins) {
-        X.wide = true;
-        nphib = 0;
+    if (kLeave && A.wide_list && nphib >= kWideMinPhi) {
+        const float in_phi = fminf(2.f * dphiw, kTwoPi) * Ld.phi_scale;
+        const float in_zr = (fminf(zc + wz, Ld.hi) - fmaxf(zc - wz, Ld.lo)) * Ld.zr_scale;
+        if (in_phi * in_zr >= A.wide_bins) {
+            X.wide = true;
+            nphib = 0;
+        }
     }
     int nlist = 0, n_compat = 0;
     // Loads run one ahead: the offsets of the next phi bin load while this
@@ -1700,9 +1726,8 @@ extern "C" mkf_status mkf_find(mkf_ctx *ctx, const mkf_hitbins *bins, const int3
     A.wide_list = leave ? tail : nullptr;
     A.wide_count = leave ? tail + n_seeds : nullptr;
     A.wide_next = leave ? tail + n_seeds + 1 : nullptr;
-    const int64_t wide_bins =
-        wide_hits(n_seeds, N, params->seed_list != nullptr) * bins->n_bins / std::max(1, bins->n_hits);
-    A.wide_bins = static_cast<int32_t>(std::min<int64_t>(std::max<int64_t>(wide_bins, 1), 1 << 30));
+    A.wide_bins = wide_bins(phys, n_seeds, N, params->seed_list != nullptr, bins->n_hits, bins->n_bins, bins->n_events,
+                            ctx->geom.n_layers);
     A.order_key = grouped ? ob : nullptr;
     A.order_pos = grouped ? ob + n_seeds : nullptr;
     int32_t *const order = grouped ? ob + 2 * (size_t)n_seeds : nullptr;
