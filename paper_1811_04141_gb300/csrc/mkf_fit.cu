@@ -115,7 +115,7 @@ struct HitRow {
 // fault and taken as no hit.
 constexpr int kFitThreads = 128;
 
-template <bool kBackward>
+template <bool kBackward, bool kAhead>
 struct HitFeed {
     const FitArgs &A;
     const int t;
@@ -145,42 +145,48 @@ struct HitFeed {
     }
     __device__ __forceinline__ HitFeed(const FitArgs &A_, int t_, float (*buf_)[4][kFitThreads])
         : A(A_), t(t_), buf(buf_) {
+        if (!kAhead) return;
         h0 = checked(index(0));
         h1 = index(1);
         copy(0, h0);
     }
+#else
+    HitFeed(const FitArgs &A_, int t_, float (*)[4][kFitThreads]) : A(A_), t(t_) {}
+#endif
     // the next row; false after the last one
     __device__ __forceinline__ bool next(HitRow &r) {
         if (kk >= A.max_hits) return false;
-        r.h = h0;
-        h0 = checked(h1);
-        copy(kk + 1, h0);
-        h1 = index(kk + 2);
-        asm volatile("cp.async.wait_group 1;" ::: "memory");
-        const float (*b)[kFitThreads] = buf[kk & 1];
-        if (r.h >= 0) {
-            r.x = b[0][threadIdx.x];
-            r.y = b[1][threadIdx.x];
-            r.z = b[2][threadIdx.x];
-            r.l = __float_as_int(b[3][threadIdx.x]);
+#ifdef __CUDACC__
+        if constexpr (kAhead) {
+            r.h = h0;
+            h0 = checked(h1);
+            copy(kk + 1, h0);
+            h1 = index(kk + 2);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+            const float (*b)[kFitThreads] = buf[kk & 1];
+            if (r.h >= 0) {
+                r.x = b[0][threadIdx.x];
+                r.y = b[1][threadIdx.x];
+                r.z = b[2][threadIdx.x];
+                r.l = __float_as_int(b[3][threadIdx.x]);
+            }
+            ++kk;
+            return true;
         }
-        ++kk;
-        return true;
-    }
-#else
-    HitFeed(const FitArgs &A_, int t_, float (*)[4][kFitThreads]) : A(A_), t(t_) {}
-    bool next(HitRow &r) {
-        if (kk >= A.max_hits) return false;
-        r.h = checked(index(kk++));
-        if (r.h >= 0) {
+#endif
+        r.h = index(kk++);
+        if (kAhead) r.h = checked(r.h);
+        else if (r.h >= A.n_hits) r.h = -1;
+#ifndef __CUDACC__
+        if (kAhead && r.h >= 0) {
+            r.l = A.hit_layer[r.h];
             r.x = A.X[r.h];
             r.y = A.Y[r.h];
             r.z = A.Z[r.h];
-            r.l = A.hit_layer[r.h];
         }
+#endif
         return true;
     }
-#endif
     // the row handed out last
     __device__ __forceinline__ int k() const { return row(kk - 1); }
 };
@@ -205,26 +211,53 @@ __device__ __forceinline__ bool first_three(const FitArgs &A, int t, int first[3
     return nfirst >= 3;
 }
 
+// Blocks of 128 tracks per SM that fit_kernel is compiled for, by physics variant
+// (see there), and the choice for a call: more blocks on an SM mean spilled
+// registers but fewer waves, and where the last wave is nearly empty that decides.
+// A wave of 4, 5 and 6 blocks costs about 16, 20 (18 backward) and 23 (a full wave,
+// material, forward / backward: 86 / 77, 108 / 91, 121 / 115 us); over many waves
+// the three come out alike and the variants without spills are taken.  With
+// the fewest blocks only, calls just above one wave took as long as two: 110 000
+// tracks of 24 rows with material 174 / 160 us, now 147 / 145 (6 blocks); 90 000
+// tracks 161 / 151 us, now 133 / 116 (5 blocks); uniform field, 110 000 tracks of 12
+// rows 77, now 69.
+constexpr int fit_blocks(int phys) { return phys == 0 ? 5 : phys == 1 ? 4 : 3; }
+
+inline int fit_blocks_for(int phys, bool backward, int blocks, int sms) {
+    int best = fit_blocks(phys);
+    if (phys == 2) return best;
+    auto waves = [&](int k) { return (blocks - 1) / (sms * k) + 1; };
+    auto cost = [&](int k) { return static_cast<int64_t>(waves(k)) * (k == 4 ? 16 : k == 5 ? (backward ? 18 : 20) : 23); };
+    if (phys == 1 && cost(5) < cost(4)) best = 5;
+    if (waves(6) <= (backward ? 1 : 3) && cost(6) < cost(best)) best = 6;
+    return best;
+}
+
 // kBackward: hits in reverse order from the given state at the last hit, turned
 // around and inflated; the result at the first hit is turned back.  kPhys: 0
 // uniform field without material; 1 material effects compiled in (selected
 // when any layer has material); 2 the parameterised field (Runge-Kutta
 // propagation) with the material effects.
 // Bound: issue and instruction fetch (the uniform-field fit: 72 % of issue slots,
-// the hit code is there twice).  Blocks per SM, measured with the row feed:
+// the hit code is there twice).  kBlocks per SM, measured with the row feed:
 // uniform field 6 / 5 / 4: 334 / 322 / 333 us for 10^6 tracks of 10 hits (at 5
 // nothing spills; 336 us before the feed, at 6); material, out and back, 6 / 5 /
 // 4 / 3: 384 / 332 / 311 / 342 us for 144 000 tracks of 16 hits (367 us before,
 // at 6, where the square root of nine columns spilled 420 bytes a thread);
 // parameterised field 4 / 3 / 2: 547 / 497 / 512 us for 10^5 tracks of 10 hits.
-template <bool kBackward, int kPhys>
-__global__ void __launch_bounds__(128, kPhys == 0 ? 5 : kPhys == 1 ? 4 : 3) fit_kernel(const __grid_constant__ FitArgs A) {
+// Which one a call gets: fit_blocks_for.  At 6 the rows are loaded where they are
+// used: the feed's registers spill (material, forward, 110 000 tracks: 167 us with
+// it, 147 without).
+template <bool kBackward, int kPhys, int kBlocks = fit_blocks(kPhys)>
+__global__ void __launch_bounds__(128, kBlocks) fit_kernel(const __grid_constant__ FitArgs A) {
     constexpr bool kMaterial = kPhys >= 1, kParamField = kPhys == 2;
+    constexpr bool kAhead = kBlocks < 6;
     constexpr int kSq = kMaterial ? 9 : 5;  // square-root columns through the seed hits
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= A.n) return;
 #ifdef __CUDACC__
-    __shared__ float buf[2][4][kFitThreads];
+    __shared__ float shared[kAhead ? 2 : 1][4][kAhead ? kFitThreads : 1];
+    float (*const buf)[4][kFitThreads] = reinterpret_cast<float (*)[4][kFitThreads]>(shared);
 #else
     float (*const buf)[4][kFitThreads] = nullptr;
 #endif
@@ -263,8 +296,8 @@ __global__ void __launch_bounds__(128, kPhys == 0 ? 5 : kPhys == 1 ? 4 : 3) fit_
             ok = seed_state(G.L[l0], kbs, h1, h2, h3, p, Q, eta);
         }
     }
-    if (!ok) {
-        st |= MKF_ST_BADSEED;
+    if (!ok) st |= MKF_ST_BADSEED;
+    if (!ok || !kAhead) {  // (else the feed reports them)
         // the list's invalid indices are reported all the same
         for (int k = 0; k < A.max_hits; ++k)
             if (A.hit_idx[(int64_t)k * A.n + t] >= A.n_hits) record_fault(A.fault, kFaultBadHitIndex, t);
@@ -275,11 +308,12 @@ __global__ void __launch_bounds__(128, kPhys == 0 ? 5 : kPhys == 1 ? 4 : 3) fit_
         // one hit: onto its layer (after the first), material, update; Cx is
         // the covariance (float[21]) or, through the seed hits, its square root
         auto hit = [&](auto Cx, const HitRow &r) {
-            if (r.l < 0 || r.l >= G.n_layers) {
+            const int l = kAhead ? r.l : A.hit_layer[r.h];
+            if (l < 0 || l >= G.n_layers) {
                 record_fault(A.fault, kFaultBadLayer, r.h);
                 return;
             }
-            const LayerDesc &Ld = G.L[r.l];
+            const LayerDesc &Ld = G.L[l];
             if (!firsthit) {
                 if (!move_to<kPhys>(G, Ld, p, lo, Cx)) {
                     st |= MKF_ST_UNREACHABLE;
@@ -294,7 +328,8 @@ __global__ void __launch_bounds__(128, kPhys == 0 ? 5 : kPhys == 1 ? 4 : 3) fit_
             }
             firsthit = false;
             float dchi2;
-            if (update_with(Ld, r.x, r.y, r.z, p, lo, Cx, dchi2)) {
+            if (update_with(Ld, kAhead ? r.x : A.X[r.h], kAhead ? r.y : A.Y[r.h], kAhead ? r.z : A.Z[r.h], p, lo, Cx,
+                            dchi2)) {
                 chi2 += dchi2;
                 ++used;
             } else {
@@ -310,7 +345,7 @@ __global__ void __launch_bounds__(128, kPhys == 0 ? 5 : kPhys == 1 ? 4 : 3) fit_
                 add_scattering(Ld.kind, mx0, p, Cx);
             }
         };
-        HitFeed<kBackward> feed(A, t, buf);
+        HitFeed<kBackward, kAhead> feed(A, t, buf);
         HitRow r;
         if constexpr (!kBackward) {
             if (!A.seed_par) {  // from the seed prior: the seed hits with the square root
@@ -706,7 +741,7 @@ __global__ void __launch_bounds__(128, 3) smooth_kernel(const __grid_constant__ 
                 st |= MKF_ST_BADS;
             }
         };
-        HitFeed<false> feed(A, t, buf);
+        HitFeed<false, true> feed(A, t, buf);
         HitRow r;
         auto row = [&](auto Cx) {
             const int k = feed.k();
@@ -834,14 +869,25 @@ static mkf_status launch_fit(mkf_ctx *ctx, const float *xyz, const int32_t *hit_
         MKF_CUDA_TRY(cudaGetLastError());
         return MKF_OK;
     }
-    switch (mkf_phys_variant(ctx->geom) + (backward ? 3 : 0)) {
-        case 0: fit_kernel<false, 0><<<blocks, threads, 0, ctx->stream>>>(A); break;
-        case 1: fit_kernel<false, 1><<<blocks, threads, 0, ctx->stream>>>(A); break;
-        case 2: fit_kernel<false, 2><<<blocks, threads, 0, ctx->stream>>>(A); break;
-        case 3: fit_kernel<true, 0><<<blocks, threads, 0, ctx->stream>>>(A); break;
-        case 4: fit_kernel<true, 1><<<blocks, threads, 0, ctx->stream>>>(A); break;
-        default: fit_kernel<true, 2><<<blocks, threads, 0, ctx->stream>>>(A); break;
+    const int phys = mkf_phys_variant(ctx->geom);
+    const int per_sm = fit_blocks_for(phys, backward, blocks, ctx->num_sms);
+    typedef void (*FitFn)(FitArgs);
+    FitFn fn;
+    switch ((phys == 2 ? 6 : phys * 3 + per_sm - 4) + (backward ? 7 : 0)) {
+        case 1: fn = fit_kernel<false, 0, 5>; break;
+        case 2: fn = fit_kernel<false, 0, 6>; break;
+        case 3: fn = fit_kernel<false, 1, 4>; break;
+        case 4: fn = fit_kernel<false, 1, 5>; break;
+        case 5: fn = fit_kernel<false, 1, 6>; break;
+        case 6: fn = fit_kernel<false, 2>; break;
+        case 8: fn = fit_kernel<true, 0, 5>; break;
+        case 9: fn = fit_kernel<true, 0, 6>; break;
+        case 10: fn = fit_kernel<true, 1, 4>; break;
+        case 11: fn = fit_kernel<true, 1, 5>; break;
+        case 12: fn = fit_kernel<true, 1, 6>; break;
+        default: fn = fit_kernel<true, 2>; break;
     }
+    fn<<<blocks, threads, 0, ctx->stream>>>(A);
     MKF_CUDA_TRY(cudaGetLastError());
     return MKF_OK;
 }
