@@ -341,15 +341,21 @@ struct Expansion {
 // times as many in the parameterised field, where a seed begun anew repeats its
 // Runge-Kutta steps (8 events with windows of most of a layer 2.40 ms, 1.87 at
 // four times, 1.85 with none left; dense events the same either way).
+// And there only in layers of 2000 hits: in smaller ones no window is worth it (an
+// event of 2000 tracks and 20 000 noise hits 0.95 ms, 0.87 with none left).
 inline int wide_hits(int phys, int n_seeds, int n_best, bool listed, bool crowded) {
     const int hits = std::min(std::max(n_seeds / (listed ? 384 : 192), n_best > 1 && crowded ? 128 : 256), 512);
     return phys == 2 ? 4 * hits : hits;
 }
 
-// The same in bins of the call's grid (each layer has its own: n_bins in all).
+// Hits of a layer in an event, on average.
+inline int layer_hits(int n_hits, int n_events, int n_layers) { return n_hits / n_layers / std::max(1, n_events); }
+constexpr int kFieldLeaveHits = 2000;
+
+// wide_hits in bins of the call's grid (each layer has its own: n_bins in all).
 inline float wide_bins(int phys, int n_seeds, int n_best, bool listed, int n_hits, int64_t n_bins, int n_events,
                        int n_layers) {
-    const bool crowded = n_hits / n_layers / std::max(1, n_events) >= 4000;
+    const bool crowded = layer_hits(n_hits, n_events, n_layers) >= 4000;
     return static_cast<float>(wide_hits(phys, n_seeds, n_best, listed, crowded)) * static_cast<float>(n_bins) /
            static_cast<float>(std::max(1, n_hits));
 }
@@ -373,8 +379,8 @@ constexpr int kWideMinPhi = 4;
 // candidate is held by `lanes` lanes, which share its window: lane `sub` takes
 // the phi bins sub, sub + lanes, ... counted from the middle of the window
 // outwards (the best hits come first and the lists settle) and keeps a list of
-// its own.
-template <int kPhys, bool kLeave, bool kShared>
+// its own.  kCols: see propagate_field.
+template <int kPhys, bool kLeave, bool kShared, int kCols>
 __device__ __forceinline__ void expand(const FindArgs &A, const Geom &G, int ev, unsigned long long mask, int dir,
                                        int N, float cut, float p[6], Lo &lo, float C[21], Book &bk, Innov &I,
                                        uint32_t &status, int &c_cl, int &c_ht, float *lchi, int *lorig, float *lu,
@@ -398,7 +404,7 @@ __device__ __forceinline__ void expand(const FindArgs &A, const Geom &G, int ev,
     }
     const LayerDesc &Ld = G.L[l];
     if (kPhys == 2)
-        propagate_field(Ld, G.kb, G.alpha, p, lo, C, sphi, cphi, -p[3] * kbl, s);
+        propagate_field<kCols>(Ld, G.kb, G.alpha, p, lo, C, sphi, cphi, -p[3] * kbl, s);
     else
         propagate_transport(Ld, G.kb, p, lo, C, sphi, cphi, cot, s);
     if (kPhys >= 1) {
@@ -517,6 +523,10 @@ __device__ __forceinline__ void expand(const FindArgs &A, const Geom &G, int ev,
 // seed's eta, the direction along z and the first layers beyond the third hit.
 // kPhys: 0 uniform field, 1 material effects, 2 parameterised field
 // (Runge-Kutta propagation) and material effects.
+// Moves in the field with all columns side by side: the kernel has the registers
+// (no spills; one event of 500 tracks 3 % faster than with the loop).
+constexpr int kSeedCols = 6;
+
 template <int kPhys>
 __global__ void __launch_bounds__(128) seed_kernel(const __grid_constant__ FindArgs A) {
     constexpr bool kParamField = kPhys == 2;
@@ -580,7 +590,7 @@ __global__ void __launch_bounds__(128) seed_kernel(const __grid_constant__ FindA
                 break;
             }
             if (kParamField)
-                propagate_field(Ld, G.kb, G.alpha, p, lo, &Q, sphi, cphi, -p[3] * kbl, s);
+                propagate_field<kSeedCols>(Ld, G.kb, G.alpha, p, lo, &Q, sphi, cphi, -p[3] * kbl, s);
             else
                 propagate_transport(Ld, G.kb, p, lo, &Q, sphi, cphi, cot, s);
             if (kPhys >= 1) {
@@ -658,7 +668,8 @@ __global__ void __launch_bounds__(128) seed_kernel(const __grid_constant__ FindA
         float lchi[MKF_MAX_NBEST], lu[MKF_MAX_NBEST], lv[MKF_MAX_NBEST];
         int lorig[MKF_MAX_NBEST];
         Expansion X;
-        expand<kPhys, false, false>(A, G, ev, mask, dir, N, A.cut, p, lo, C, bk, I, status, c_cl, c_ht, lchi, lorig, lu, lv, 1, X);
+        expand<kPhys, false, false, kSeedCols>(A, G, ev, mask, dir, N, A.cut, p, lo, C, bk, I, status, c_cl, c_ht, lchi,
+                                               lorig, lu, lv, 1, X);
         nlist = X.nlist;
         searched = X.searched;
         nbeam = min(searched ? nlist + 1 : 1, N);
@@ -765,7 +776,9 @@ __device__ __forceinline__ void write_track(const FindArgs &A, int seed, int ev,
 // kN: the beam width N fixed at compile time (1 or 10, the widths the finder
 // mostly runs with: the segment loops and lane arithmetic fold, 3-4 % faster;
 // not for the parameterised field), or 0 for N taken from the arguments.
-template <bool kLearned, int kPhys, int kN>
+// kCols: the columns of a move in the parameterised field side by side (see
+// propagate_field; mkf_find chooses).
+template <bool kLearned, int kPhys, int kN, int kCols = 1>
 __global__ void __launch_bounds__(256, 2) find_kernel(const __grid_constant__ FindArgs A) {
     // (learned: the cascade's best-hit pass)
     constexpr bool kLeave = kPhys >= 1 && (!kLearned || kN == 1);
@@ -963,8 +976,8 @@ __global__ void __launch_bounds__(256, 2) find_kernel(const __grid_constant__ Fi
             // ---- 1. expansion: next layer, propagation, window search
             Expansion X{-1, false, 0, 0, 0.f, false};
             if (active) {
-                expand<kPhys, kLeave, false>(A, G, ev, mask, dir, N, cut, p, lo, C, bk, I, status, c_cl, c_ht,
-                                             lchi + lane, lorig + lane, lu + lane, lv + lane, 32, X);
+                expand<kPhys, kLeave, false, kCols>(A, G, ev, mask, dir, N, cut, p, lo, C, bk, I, status, c_cl, c_ht,
+                                                    lchi + lane, lorig + lane, lu + lane, lv + lane, 32, X);
             }
             if (kLeave && A.wide_list) {
                 // a seed with a wide window ends here, without output: it is
@@ -1435,7 +1448,7 @@ __global__ void __launch_bounds__(256, 2) find_wide_kernel(const __grid_constant
             if (!__syncthreads_or(active)) break;
             Expansion X{-1, false, 0, 0, 0.f, false};
             if (active)
-                expand<kPhys, false, true>(A, G, ev, mask, dir, N, cut, p, lo, C, bk, I, status, c_cl, c_ht,
+                expand<kPhys, false, true, 1>(A, G, ev, mask, dir, N, cut, p, lo, C, bk, I, status, c_cl, c_ht,
                                            lchi + tid, lorig + tid, lu + tid, lv + tid, nt, X, sub, lanes);
             // the candidate's list from its lanes' lists: the smallest remaining
             // (chi2, hit index) of the lanes' heads, N times
@@ -1663,6 +1676,7 @@ extern "C" mkf_status mkf_find(mkf_ctx *ctx, const mkf_hitbins *bins, const int3
         reinterpret_cast<const void *>(find_kernel<true, 1, 10>), reinterpret_cast<const void *>(find_kernel<true, 2, 0>),
         reinterpret_cast<const void *>(find_kernel<true, 2, 0>), reinterpret_cast<const void *>(find_kernel<true, 2, 0>)};
     const void *kfn = kfns[vi];
+    const void *const kfn_side = reinterpret_cast<const void *>(find_kernel<false, 2, 0, 6>);
     const void *const wfns[3] = {reinterpret_cast<const void *>(find_wide_kernel<false, 1>),
                                  reinterpret_cast<const void *>(find_wide_kernel<false, 2>),
                                  reinterpret_cast<const void *>(find_wide_kernel<true, 1>)};
@@ -1675,6 +1689,8 @@ extern "C" mkf_status mkf_find(mkf_ctx *ctx, const mkf_hitbins *bins, const int3
         for (int v = 0; v < 18; ++v)
             MKF_CUDA_TRY(cudaFuncSetAttribute(kfns[v], cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               static_cast<int>(kFindMaxSmem)));
+        MKF_CUDA_TRY(cudaFuncSetAttribute(kfn_side, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          static_cast<int>(kFindMaxSmem)));
         for (const void *w : wfns)
             MKF_CUDA_TRY(cudaFuncSetAttribute(w, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                               static_cast<int>(wide_smem_bytes(MKF_MAX_LAYERS, MKF_MAX_NBEST))));
@@ -1693,8 +1709,13 @@ extern "C" mkf_status mkf_find(mkf_ctx *ctx, const mkf_hitbins *bins, const int3
         ctx->find_occ_smem[vi] = static_cast<int>(smem);
         ctx->find_occ_blocks[vi] = occ;
     }
-    const int per_sm = ctx->find_occ_blocks[vi];
-    const int blocks = std::max(1, std::min(need, std::max(1, per_sm) * ctx->num_sms));
+    const int most = std::max(1, ctx->find_occ_blocks[vi]) * ctx->num_sms;
+    const int blocks = std::max(1, std::min(need, most));
+    // in the parameterised field a call that fills half of the chip at most takes
+    // the columns of a move side by side (500 seeds 0.216 -> 0.193 ms, 4000 seeds at
+    // N = 1 0.317 -> 0.282; above the line they get slower: 16 000 at N = 4 0.47 ->
+    // 0.49, with 500 of 608 blocks)
+    if (!learned && phys == 2 && 2 * static_cast<int64_t>(need) <= most) kfn = kfn_side;
     // seeds that all have a warp at once are taken in the input order: nothing
     // waits behind a long one there, and the two kernels that make the order
     // would only come on top (2000 seeds: 79 us with them, 67 without; at the
@@ -1712,7 +1733,9 @@ extern "C" mkf_status mkf_find(mkf_ctx *ctx, const mkf_hitbins *bins, const int3
     const size_t order_bytes = grouped ? ((sizeof(int32_t) * 3 * (size_t)n_seeds + 255) / 256) * 256 : 0;
     // seeds with a wide window go to find_wide_kernel: with material, in the
     // plain finder and in the cascade's best-hit pass
-    const bool leave = learned ? phys == 1 && params->mlp_mode == 1 && N == 1 : phys >= 1;
+    const bool leave = learned ? phys == 1 && params->mlp_mode == 1 && N == 1
+                               : phys == 1 || (phys == 2 && layer_hits(bins->n_hits, bins->n_events,
+                                                                       ctx->geom.n_layers) >= kFieldLeaveHits);
     // words that start at zero: the list of those seeds and its counters, the
     // order's key counts (and their total)
     const size_t zero_words = leave ? (size_t)n_seeds + 2 : 0;

@@ -577,6 +577,7 @@ __device__ __forceinline__ void tangent_rhs(const RkStage &S, float kba, float l
 // (x, y, z, q/pT, phi, theta), whose lambda derivatives are dl.
 // d is the displacement from r0, dlo the rounding error of its updates (a
 // float pair, as the state's positions).
+template <int kCols>
 __device__ __forceinline__ void rk_step(float kb, float alpha, const float r0[3], float lam, const float dl[6],
                                         float d[3], float dlo[3], float T[3], float Dr[6][3], float DT[6][3],
                                         float hs) {
@@ -614,7 +615,7 @@ __device__ __forceinline__ void rk_step(float kb, float alpha, const float r0[3]
         T[i] = fmaf(h6 * lam, st[i] + S[3].tb[i], T[i]);
     }
     const float kba = kb * alpha;
-#pragma unroll 1  // one column's code, see move_field
+#pragma unroll kCols  // see propagate_field
     for (int c = 0; c < 6; ++c) {
         float ar[3], at[3], ir[3], it[3], k[3];
         // stage 1
@@ -675,15 +676,9 @@ __device__ __forceinline__ float nearest_root(float a, float b, float c) {
 // parameter columns (dr, dT) integrated with the trajectory (the variational
 // equations, the field's gradient included), then the surface constraint
 // dS = -(n . dr) / (n . T) moves every column along (T, dT/dS) at the end.
-// The code of this function is long, and fetching it was what bounded the
-// kernels in the field: the fit of 10^5 tracks of 10 hits took 866 us with two
-// copies of rk_step and six unrolled columns inlined for either covariance form,
-// 610 us with one copy of rk_step, 489 us with the columns in a loop as well
-// (their arrays then lie in local memory, which the first-level cache holds), 497
-// us as it is now, called instead of inlined (which keeps every bit of the
-// results, the inlined form did not).
-MKF_CALLED void move_field(const LayerDesc &Ld, float kb, float alpha, float p[6], Lo &lo,
-                                        float (&J)[6][6], float sphi, float cphi, float h, float s) {
+template <int kCols>
+__device__ __forceinline__ void move_in_field(const LayerDesc &Ld, float kb, float alpha, float p[6], Lo &lo,
+                                              float (&J)[6][6], float sphi, float cphi, float h, float s) {
     float st, ct;
     sincos_pair(p[5], lo.th, st, ct);
     const float lam = p[3] * st;
@@ -723,7 +718,7 @@ MKF_CALLED void move_field(const LayerDesc &Ld, float kb, float alpha, float p[6
                 dn = ((Ld.rz - p[2]) - ((lo.z + dlo[2]) + d[2])) / T[2];
             }
         }
-        rk_step(kb, alpha, r0, lam, dl, d, dlo, T, Dr, DT, dn);
+        rk_step<kCols>(kb, alpha, r0, lam, dl, d, dlo, T, Dr, DT, dn);
     }
 
     // end point: dT/dS, surface normal, output conversions
@@ -784,11 +779,31 @@ MKF_CALLED void move_field(const LayerDesc &Ld, float kb, float alpha, float p[6
     p[3] = lam / sth;
 }
 
-template <class Cov>
+// The same, called.
+template <int kCols>
+MKF_CALLED void call_move_in_field(const LayerDesc &Ld, float kb, float alpha, float p[6], Lo &lo, float (&J)[6][6],
+                                   float sphi, float cphi, float h, float s) {
+    move_in_field<kCols>(Ld, kb, alpha, p, lo, J, sphi, cphi, h, s);
+}
+
+// The code of a move is long, and fetching it is what bounds the kernels in the
+// field when the chip is full: the fit of 10^5 tracks of 10 hits took 866 us with
+// two copies of rk_step and six unrolled columns inlined for either covariance
+// form, 610 us with one copy of rk_step, 489 us with the columns in a loop as well
+// (their arrays then lie in local memory, which the first-level cache holds), 497
+// us called instead of inlined (which keeps every bit of the results, the inlined
+// loop did not).  In small calls the chain of one column after the other bounds
+// instead: finding in one event of 500 tracks took 7 % longer with the loop than
+// with the six columns side by side.  kCols columns side by side: 1 or 2 called, 6
+// inlined (all three the same bits).  Each kernel's choice stands where it is made.
+template <int kCols, class Cov>
 __device__ __forceinline__ void propagate_field(const LayerDesc &Ld, float kb, float alpha, float p[6], Lo &lo,
                                                 Cov C, float sphi, float cphi, float h, float s) {
     float J[6][6];
-    move_field(Ld, kb, alpha, p, lo, J, sphi, cphi, h, s);
+    if constexpr (kCols == 6)
+        move_in_field<kCols>(Ld, kb, alpha, p, lo, J, sphi, cphi, h, s);
+    else
+        call_move_in_field<kCols>(Ld, kb, alpha, p, lo, J, sphi, cphi, h, s);
     transport_cov(J, C);
 }
 
