@@ -246,10 +246,10 @@ inline int fit_blocks_for(int phys, bool backward, int blocks, int sms) {
 // 4 / 3: 384 / 332 / 311 / 342 us for 144 000 tracks of 16 hits (367 us before,
 // at 6, where the square root of nine columns spilled 420 bytes a thread);
 // parameterised field 4 / 3 / 2: 547 / 497 / 512 us for 10^5 tracks of 10 hits.
-// Which one a call gets: fit_blocks_for.  At 6 the rows are loaded where they are
+// Which one a call gets: fit_blocks_for.  kCols: see propagate_field.  At 6 the rows are loaded where they are
 // used: the feed's registers spill (material, forward, 110 000 tracks: 167 us with
 // it, 147 without).
-template <bool kBackward, int kPhys, int kBlocks = fit_blocks(kPhys)>
+template <bool kBackward, int kPhys, int kBlocks = fit_blocks(kPhys), int kCols = 1>
 __global__ void __launch_bounds__(128, kBlocks) fit_kernel(const __grid_constant__ FitArgs A) {
     constexpr bool kMaterial = kPhys >= 1, kParamField = kPhys == 2;
     constexpr bool kAhead = kBlocks < 6;
@@ -316,9 +316,7 @@ __global__ void __launch_bounds__(128, kBlocks) fit_kernel(const __grid_constant
             }
             const LayerDesc &Ld = G.L[l];
             if (!firsthit) {
-                // columns: forward 2 / 1 at a time 155 / 161 us for 1000 tracks, 501 / 505
-                // for 90 000; backward 155 / 151, 456 / 471
-                if (!move_to<kPhys, kBackward ? 1 : 2>(G, Ld, p, lo, Cx)) {
+                if (!move_to<kPhys, kCols>(G, Ld, p, lo, Cx)) {
                     st |= MKF_ST_UNREACHABLE;
                     return;
                 }
@@ -882,7 +880,12 @@ static mkf_status launch_fit(mkf_ctx *ctx, const float *xyz, const int32_t *hit_
         case 3: fn = fit_kernel<false, 1, 4>; break;
         case 4: fn = fit_kernel<false, 1, 5>; break;
         case 5: fn = fit_kernel<false, 1, 6>; break;
-        case 6: fn = fit_kernel<false, 2>; break;
+        case 6:
+            // forward in the field, up to a wave: two columns of a move at a time (1000
+            // tracks 161 -> 155 us, 38 000 241 -> 237; 100 000 500 -> 506; backward the
+            // other way round: 151 -> 155 us for 1000)
+            fn = blocks <= fit_blocks(2) * ctx->num_sms ? fit_kernel<false, 2, fit_blocks(2), 2> : fit_kernel<false, 2>;
+            break;
         case 8: fn = fit_kernel<true, 0, 5>; break;
         case 9: fn = fit_kernel<true, 0, 6>; break;
         case 10: fn = fit_kernel<true, 1, 4>; break;
