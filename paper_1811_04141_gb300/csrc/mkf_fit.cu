@@ -111,8 +111,9 @@ struct HitRow {
 // earlier still: the gathers (four of them behind an index load, 700 cycles
 // each from L2) then cost the filter no wait, and no registers (prefetched into
 // registers they spilled and gained nothing).  The kernel of one event of 1000
-// tracks went from 20.5 to 17.3 us; for 10^6 tracks see fit_kernel.  Every
-// thread waits for its own copies only.  An index outside [0, n_hits) is a device
+// tracks went from 20.5 to 17.3 us (a call takes 23 as before: the host's part
+// is longer); for 10^6 tracks see fit_kernel.  Every thread waits for its own
+// copies only.  An index outside [0, n_hits) is a device
 // fault and taken as no hit.
 constexpr int kFitThreads = 128;
 
@@ -215,13 +216,14 @@ __device__ __forceinline__ bool first_three(const FitArgs &A, int t, int first[3
 // Blocks of 128 tracks per SM that fit_kernel is compiled for, by physics variant
 // (see there), and the choice for a call: more blocks on an SM mean spilled
 // registers but fewer waves, and where the last wave is nearly empty that decides.
-// A wave of 4, 5 and 6 blocks costs about 16, 20 (18 backward) and 23 (a full wave,
-// material, forward / backward: 86 / 77, 108 / 91, 121 / 115 us); over many waves
-// the three come out alike and the variants without spills are taken.  With
-// the fewest blocks only, calls just above one wave took as long as two: 110 000
-// tracks of 24 rows with material 174 / 160 us, now 147 / 145 (6 blocks); 90 000
-// tracks 161 / 151 us, now 133 / 116 (5 blocks); uniform field, 110 000 tracks of 12
-// rows 77, now 69.
+// A wave of 4, 5 and 6 blocks costs about 16, 18 (backward) and 23 (a full wave,
+// material, forward / backward: 86 / 77, - / 91, 121 / 115 us); over many waves
+// they come out alike and the variants without spills are taken.  With the
+// fewest blocks only, calls just above one wave took as long as two: 110 000
+// tracks of 24 rows with material 146 / 131 us, now 121 / 116 (6 blocks); 90 000
+// tracks 135 / 121 us, now 106 / 89 (6 / 5 blocks); uniform field, 110 000 tracks
+// of 12 rows 54, now 46.  Forward with material 5 blocks are never the best by
+// more than 3 %.
 constexpr int fit_blocks(int phys) { return phys == 0 ? 5 : phys == 1 ? 4 : 3; }
 
 inline int fit_blocks_for(int phys, bool backward, int blocks, int sms) {
@@ -229,7 +231,7 @@ inline int fit_blocks_for(int phys, bool backward, int blocks, int sms) {
     if (phys == 2) return best;
     auto waves = [&](int k) { return (blocks - 1) / (sms * k) + 1; };
     auto cost = [&](int k) { return static_cast<int64_t>(waves(k)) * (k == 4 ? 16 : k == 5 ? (backward ? 18 : 20) : 23); };
-    if (phys == 1 && cost(5) < cost(4)) best = 5;
+    if (phys == 1 && backward && cost(5) < cost(4)) best = 5;
     if (waves(6) <= (backward ? 1 : 3) && cost(6) < cost(best)) best = 6;
     return best;
 }
@@ -247,8 +249,7 @@ inline int fit_blocks_for(int phys, bool backward, int blocks, int sms) {
 // at 6, where the square root of nine columns spilled 420 bytes a thread);
 // parameterised field 4 / 3 / 2: 547 / 497 / 512 us for 10^5 tracks of 10 hits.
 // Which one a call gets: fit_blocks_for.  kCols: see propagate_field.  At 6 the rows are loaded where they are
-// used: the feed's registers spill (material, forward, 110 000 tracks: 167 us with
-// it, 147 without).
+// used: the feed's registers spill (material, forward, 110 000 tracks: 13 % slower).
 template <bool kBackward, int kPhys, int kBlocks = fit_blocks(kPhys), int kCols = 1>
 __global__ void __launch_bounds__(128, kBlocks) fit_kernel(const __grid_constant__ FitArgs A) {
     constexpr bool kMaterial = kPhys >= 1, kParamField = kPhys == 2;
@@ -878,7 +879,6 @@ static mkf_status launch_fit(mkf_ctx *ctx, const float *xyz, const int32_t *hit_
         case 1: fn = fit_kernel<false, 0, 5>; break;
         case 2: fn = fit_kernel<false, 0, 6>; break;
         case 3: fn = fit_kernel<false, 1, 4>; break;
-        case 4: fn = fit_kernel<false, 1, 5>; break;
         case 5: fn = fit_kernel<false, 1, 6>; break;
         case 6:
             // forward in the field, up to a wave: two columns of a move at a time (1000
