@@ -81,7 +81,7 @@ struct mkf_hitbins {
 // Launch of a kernel that starts with after_previous(): a programmatic dependent
 // launch, which is prepared while the stream's previous kernel runs.  A chain of
 // short kernels then does not pay each launch's latency: binning and finding of
-// one event of 2000 tracks 99 -> 80 us (with the order kernels left out of a call
+// one event of 2000 tracks 98 -> 76 us (with the order kernels left out of a call
 // that small), the chain of twenty kernels around finding on 20 such events 517
 // -> 479 us.
 template <typename... P, typename... A>
