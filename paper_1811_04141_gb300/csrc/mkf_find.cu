@@ -335,16 +335,19 @@ struct Expansion {
 // 0.91, 0.91, 0.99; 2.0).  A call on a list of seeds knows its length on the device
 // only and is taken to work on half (a cascade's second pass over 16 such events:
 // 250 hits 2.2 ms, 500 2.4; over 96: 8.4 and 7.9).
-// 128 hits only where a layer holds 4000 (crowded): in one of 1000 they are as
-// wide as it gets, and the seed is begun anew for nothing (4 events of 2000 tracks
-// and 20 000 noise hits 0.84 ms at 128, 0.73 at 256; 0.80 with none left).  Four
+// 128 hits only where an event's layer holds 4000 of them, or no more than 400: in
+// between (a third of the layer, 256 at most) many seeds have one such window
+// and are begun anew for nothing (4 events of 2000 tracks and 20 000 noise hits,
+// 1150 a layer: 0.84 ms at 128, 0.73 at 256, 0.80 with none left; 16 of 1000 and
+// 1000, 380 a layer, a third of their seeds: 0.44, 0.48, 0.53).  Four
 // times as many in the parameterised field, where a seed begun anew repeats its
 // Runge-Kutta steps (8 events with windows of most of a layer 2.40 ms, 1.87 at
 // four times, 1.85 with none left; dense events the same either way).
 // And there only in layers of 2000 hits: in smaller ones no window is worth it (an
 // event of 2000 tracks and 20 000 noise hits 0.95 ms, 0.87 with none left).
-inline int wide_hits(int phys, int n_seeds, int n_best, bool listed, bool crowded) {
-    const int hits = std::min(std::max(n_seeds / (listed ? 384 : 192), n_best > 1 && crowded ? 128 : 256), 512);
+inline int wide_hits(int phys, int n_seeds, int n_best, bool listed, int in_layer) {
+    const int least = n_best == 1 ? 256 : in_layer >= 4000 ? 128 : std::min(std::max(in_layer / 3, 128), 256);
+    const int hits = std::min(std::max(n_seeds / (listed ? 384 : 192), least), 512);
     return phys == 2 ? 4 * hits : hits;
 }
 
@@ -355,9 +358,8 @@ constexpr int kFieldLeaveHits = 2000;
 // wide_hits in bins of the call's grid (each layer has its own: n_bins in all).
 inline float wide_bins(int phys, int n_seeds, int n_best, bool listed, int n_hits, int64_t n_bins, int n_events,
                        int n_layers) {
-    const bool crowded = layer_hits(n_hits, n_events, n_layers) >= 4000;
-    return static_cast<float>(wide_hits(phys, n_seeds, n_best, listed, crowded)) * static_cast<float>(n_bins) /
-           static_cast<float>(std::max(1, n_hits));
+    const int hits = wide_hits(phys, n_seeds, n_best, listed, layer_hits(n_hits, n_events, n_layers));
+    return static_cast<float>(hits) * static_cast<float>(n_bins) / static_cast<float>(std::max(1, n_hits));
 }
 
 // A window is measured by its own extent and not by the bins it touches: on a
